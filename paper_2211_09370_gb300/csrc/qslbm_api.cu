@@ -756,7 +756,7 @@ int create_impl(const qslbm_params* pin, qslbm_handle** out) {
         }
     }
     if (s.resident) {
-        const size_t xb = (size_t)2 * 3 * s.n * s.esz;
+        const size_t xb = (size_t)2 * (s.esz == 8 ? 5 : 3) * s.n * s.esz;
         const size_t sb = sizeof(unsigned int) * (4 + (size_t)s.nz);
         if ((rc = dev_alloc(s, &s.xbuf, xb))) goto fail;
         if ((rc = dev_alloc(s, &s.rsync, sb))) goto fail;

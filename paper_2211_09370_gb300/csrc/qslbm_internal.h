@@ -104,7 +104,10 @@ struct State {
     int ib_staged_u = 1;        // its shell nodes per thread per batch of loads (1, 2 or 5)
     bool resident_uhalo = false;
     size_t resident_smem = 0;
-    void* xbuf = nullptr;   // [2][nz][3][P] plane exchange
+    // FP64 2-D resident kernel: CTAs of its cluster (0: not used), rows per CTA,
+    // largest band's markers, shell nodes and list entries
+    int c2_ctas = 0, c2_rows = 0, c2_mk = 0, c2_sh = 0, c2_nnz = 0;
+    void* xbuf = nullptr;   // plane exchange, 2 parities x nz planes x 3 (FP64: 5) values a node
     void* rsync = nullptr;  // ResidentSync + flags[nz]
     int graph_steps = 0;
     // fused sweep + IB (FP32 planes beyond the resident kernel): bands of

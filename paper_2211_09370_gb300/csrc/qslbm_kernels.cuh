@@ -133,6 +133,10 @@ __device__ __forceinline__ void bext_add_xy(const T* bxy, int P, int p, T out[3]
     }
 }
 
+// w f + a in one rounding, in either precision.
+__device__ __forceinline__ float fma_rn(float w, float f, float a) { return __fmaf_rn(w, f, a); }
+__device__ __forceinline__ double fma_rn(double w, double f, double a) { return __fma_rn(w, f, a); }
+
 // ---------------------------------------------------------------------------
 // IB corrector on plane z of field f[3] (f[c] + k), run by a whole CTA after
 // the plane's predictor values are written.  sdelta: shared [3 * ring size].
@@ -149,9 +153,9 @@ __device__ __forceinline__ void ib_plane(const IBView<T>& ib, T* f0, T* f1, T* f
         for (int j = 0; j < 9; ++j) {
             const T w = ib.mk_w[9 * m + j];
             const long long q = plane_base + ib.mk_q[9 * m + j];
-            a0 += w * f0[q];
-            a1 += w * f1[q];
-            a2 += w * f2[q];
+            a0 = fma_rn(w, f0[q], a0);
+            a1 = fma_rn(w, f1[q], a1);
+            a2 = fma_rn(w, f2[q], a2);
         }
         const T s = ib.mk_s[m];
         const int l = m - m0;
@@ -167,9 +171,9 @@ __device__ __forceinline__ void ib_plane(const IBView<T>& ib, T* f0, T* f1, T* f
         for (int e = e0; e < e1; ++e) {
             const T w = ib.csr_w[e];
             const int l = ib.csr_m[e];
-            c0 += w * sdelta[3 * l + 0];
-            c1 += w * sdelta[3 * l + 1];
-            c2 += w * sdelta[3 * l + 2];
+            c0 = fma_rn(w, sdelta[3 * l + 0], c0);
+            c1 = fma_rn(w, sdelta[3 * l + 1], c1);
+            c2 = fma_rn(w, sdelta[3 * l + 2], c2);
         }
         const long long q = plane_base + ib.shell_xy[s];
         f0[q] += c0;
@@ -338,7 +342,7 @@ __device__ __forceinline__ void march_halo(int hid, int x0, int y0, int nx, int 
 //   D_z = e2(-x) - e2(+x) + e3(-y) - e3(+y),
 // where D_a = sum_b [Phi_ab(x - e_b) - Phi_ab(x + e_b)] as in sweep_node.
 // node_emf turns a node's (b, u) into (b, e) in place.
-// The EMF form is the FP32 path; its roundings are spelled out (fused
+// Its roundings are spelled out (fused
 // multiply-adds where written, nothing left to contraction) so that every
 // kernel using it (march_tile, the node-pair sweep, the batched sweep)
 // produces bitwise the same values.
@@ -355,19 +359,30 @@ __device__ __forceinline__ float emf_update(float w0, float w1, float w1k, float
     return __fmaf_rn(w0, b, __fmaf_rn(w1k, d, __fmul_rn(w1, s)));
 }
 
+// The same in FP64: 9 operations for e and 3 per component for the update.
+__device__ __forceinline__ void node_emf(double r[6], const double be[3], double sq) {
+    const double B0 = __fma_rn(sq, r[0], be[0]), B1 = __fma_rn(sq, r[1], be[1]), B2 = __fma_rn(sq, r[2], be[2]);
+    const double u0 = r[3], u1 = r[4], u2 = r[5];
+    r[3] = __fma_rn(u0, B1, -__dmul_rn(u1, B0));
+    r[4] = __fma_rn(u0, B2, -__dmul_rn(u2, B0));
+    r[5] = __fma_rn(u1, B2, -__dmul_rn(u2, B1));
+}
+__device__ __forceinline__ double emf_update(double w0, double w1, double w1k, double b, double s, double d) {
+    return __fma_rn(w0, b, __fma_rn(w1k, d, __dmul_rn(w1, s)));
+}
+
 // Shared tile of one march plane: six fields of (TY + 2) x (kMarchTX + 2)
 // cells, the tile and its one-cell halo.
 template <typename T, int TY = kMarchTY>
 using MarchTile = T[6][TY + 2][kMarchTX + 2];
 
-// The sweep over one tile and z chunk, one node per thread.  FP32 (EMF form):
+// The sweep over one tile and z chunk, one node per thread, in the EMF form:
 // each node's (e1, e2, e3) is formed once, where its (b, u) is loaded, and the
-// tile and the column registers hold (b, e); about half the arithmetic and
-// shared-memory traffic of forming the flux per neighbour, the same sweep up
-// to the order of rounding.  FP64 (direct form): the tile holds (b, u) and
-// every neighbour's flux is formed as in sweep_node, with the same
-// expressions and neighbour order, so that it rounds like the other FP64 sweep
-// kernels.  The column's plane z + 2 is loaded one plane ahead of its use.
+// tile and the column registers hold (b, e).  That is about half the FP32
+// arithmetic and shared-memory traffic of forming the flux per neighbour, the
+// same sweep up to the order of rounding; in FP64, whose rate is 1/64 of
+// FP32's and bounds the sweep, it is 42 operations a node instead of about
+// 135.  The column's plane z + 2 is loaded one plane ahead of its use.
 // TY: rows of the tile (the CTA has kMarchTX * TY threads); the results do not
 // depend on it.
 template <typename T, bool XY = true, int TY = kMarchTY>
@@ -375,7 +390,6 @@ __device__ __forceinline__ void march_tile(const Geo& g, const T* __restrict__ b
                                            const T* __restrict__ u, const SweepCoef<T>& c, int bx, int by, int bz,
                                            int chunk, MarchTile<T, TY>& tile) {
     static_assert(kMarchTX * TY >= 2 * (kMarchTX + 2) + 2 * TY, "every halo cell needs a thread");
-    constexpr bool EMF = sizeof(T) == 4;
     const int nx = g.nx, ny = g.ny, nz = g.nz;
     const int n = (int)g.n, P = nx * ny;
     const int tx = threadIdx.x % kMarchTX, ty = threadIdx.x / kMarchTX;
@@ -390,8 +404,8 @@ __device__ __forceinline__ void march_tile(const Geo& g, const T* __restrict__ b
     const T* src[6] = {bin, bin + n, bin + 2 * n, u, u + n, u + 2 * n};
     int hx, hy, hp;
     march_halo<TY>(threadIdx.x, x0, y0, nx, ny, hx, hy, hp);
-    // prv / cur / nxt: the column at z - 1, z, z + 1 ((b, e) or (b, u)); ahd:
-    // raw (b, u) of plane z + 2
+    // prv / cur / nxt: the column's (b, e) at z - 1, z, z + 1; ahd: raw (b, u)
+    // of plane z + 2
     T prv[6], cur[6], nxt[6], ahd[6];
     {
         const int zm = wrap_dec(z0, nz), zn = wrap_inc(z0, nz);
@@ -401,18 +415,16 @@ __device__ __forceinline__ void march_tile(const Geo& g, const T* __restrict__ b
             cur[v] = src[v][z0 * P + p];
             nxt[v] = src[v][zn * P + p];
         }
-        if constexpr (EMF) {
-            T be[3];
-            bext_at(c.bext_z, c.be, zm, be);
-            if constexpr (XY) bext_add_xy(c.bext_xy, P, p, be);
-            node_emf(prv, be, c.sq);
-            bext_at(c.bext_z, c.be, z0, be);
-            if constexpr (XY) bext_add_xy(c.bext_xy, P, p, be);
-            node_emf(cur, be, c.sq);
-            bext_at(c.bext_z, c.be, zn, be);
-            if constexpr (XY) bext_add_xy(c.bext_xy, P, p, be);
-            node_emf(nxt, be, c.sq);
-        }
+        T be[3];
+        bext_at(c.bext_z, c.be, zm, be);
+        if constexpr (XY) bext_add_xy(c.bext_xy, P, p, be);
+        node_emf(prv, be, c.sq);
+        bext_at(c.bext_z, c.be, z0, be);
+        if constexpr (XY) bext_add_xy(c.bext_xy, P, p, be);
+        node_emf(cur, be, c.sq);
+        bext_at(c.bext_z, c.be, zn, be);
+        if constexpr (XY) bext_add_xy(c.bext_xy, P, p, be);
+        node_emf(nxt, be, c.sq);
     }
     const T w1k = c.w1 * c.kappa;
     for (int z = z0; z < z1; ++z) {
@@ -429,12 +441,10 @@ __device__ __forceinline__ void march_tile(const Geo& g, const T* __restrict__ b
             T r[6];
 #pragma unroll
             for (int v = 0; v < 6; ++v) r[v] = src[v][z * P + hp];
-            if constexpr (EMF) {
-                T be[3];
-                bext_at(c.bext_z, c.be, z, be);
-                if constexpr (XY) bext_add_xy(c.bext_xy, P, hp, be);
-                node_emf(r, be, c.sq);
-            }
+            T be[3];
+            bext_at(c.bext_z, c.be, z, be);
+            if constexpr (XY) bext_add_xy(c.bext_xy, P, hp, be);
+            node_emf(r, be, c.sq);
 #pragma unroll
             for (int v = 0; v < 6; ++v) tile[v][hy][hx] = r[v];
         }
@@ -442,63 +452,18 @@ __device__ __forceinline__ void march_tile(const Geo& g, const T* __restrict__ b
         if (active) {
             const int cx = tx + 1, cy = ty + 1;
             const int k = z * P + p;
-            if constexpr (EMF) {
-                T s[3];
+            T s[3];
 #pragma unroll
-                for (int a = 0; a < 3; ++a)
-                    s[a] = (tile[a][cy][cx - 1] + tile[a][cy][cx + 1]) + (tile[a][cy - 1][cx] + tile[a][cy + 1][cx]) +
-                           (prv[a] + nxt[a]);
-                const T dx = (tile[3][cy + 1][cx] - tile[3][cy - 1][cx]) + (nxt[4] - prv[4]);
-                const T dy = (tile[3][cy][cx - 1] - tile[3][cy][cx + 1]) + (nxt[5] - prv[5]);
-                const T dz =
-                    (tile[4][cy][cx - 1] - tile[4][cy][cx + 1]) + (tile[5][cy - 1][cx] - tile[5][cy + 1][cx]);
-                bout[k] = emf_update(c.w0, c.w1, w1k, cur[0], s[0], dx);
-                bout[k + n] = emf_update(c.w0, c.w1, w1k, cur[1], s[1], dy);
-                bout[k + 2 * n] = emf_update(c.w0, c.w1, w1k, cur[2], s[2], dz);
-            } else {
-                T be_c[3], be_m[3], be_p[3];
-                bext_at(c.bext_z, c.be, z, be_c);
-                bext_at(c.bext_z, c.be, wrap_dec(z, nz), be_m);
-                bext_at(c.bext_z, c.be, zn, be_p);
-                T acc[3] = {c.w0 * cur[0], c.w0 * cur[1], c.w0 * cur[2]};
-                T diff[3] = {T(0), T(0), T(0)};
-#pragma unroll
-                for (int d = 0; d < 6; ++d) {
-                    T bq[3], uq[3];
-                    if (d < 4) {
-                        const int ix = cx + (d == 0 ? -1 : d == 1 ? 1 : 0);
-                        const int iy = cy + (d == 2 ? -1 : d == 3 ? 1 : 0);
-#pragma unroll
-                        for (int a = 0; a < 3; ++a) {
-                            bq[a] = tile[a][iy][ix];
-                            uq[a] = tile[3 + a][iy][ix];
-                        }
-                    } else {
-#pragma unroll
-                        for (int a = 0; a < 3; ++a) {
-                            bq[a] = d == 4 ? prv[a] : nxt[a];
-                            uq[a] = d == 4 ? prv[3 + a] : nxt[3 + a];
-                        }
-                    }
-                    const T* bez = (d < 4) ? be_c : (d == 4 ? be_m : be_p);
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) acc[a] += c.w1 * bq[a];
-                    T Bx[3] = {bez[0], bez[1], bez[2]};
-                    if constexpr (XY) {
-                        if (c.bext_xy) {
-                            const int xq = d == 0 ? wrap_dec(xc, nx) : d == 1 ? wrap_inc(xc, nx) : xc;
-                            const int yq = d == 2 ? wrap_dec(yc, ny) : d == 3 ? wrap_inc(yc, ny) : yc;
-                            bext_add_xy(c.bext_xy, P, yq * nx + xq, Bx);
-                        }
-                    }
-                    T B[3];
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) B[a] = Bx[a] + c.sq * bq[a];
-                    flux_acc(uq, B, d >> 1, (d & 1) ? T(-1) : T(1), diff);
-                }
-#pragma unroll
-                for (int a = 0; a < 3; ++a) bout[k + a * n] = acc[a] + c.w1 * c.kappa * diff[a];
-            }
+            for (int a = 0; a < 3; ++a)
+                s[a] = (tile[a][cy][cx - 1] + tile[a][cy][cx + 1]) + (tile[a][cy - 1][cx] + tile[a][cy + 1][cx]) +
+                       (prv[a] + nxt[a]);
+            const T dx = (tile[3][cy + 1][cx] - tile[3][cy - 1][cx]) + (nxt[4] - prv[4]);
+            const T dy = (tile[3][cy][cx - 1] - tile[3][cy][cx + 1]) + (nxt[5] - prv[5]);
+            const T dz =
+                (tile[4][cy][cx - 1] - tile[4][cy][cx + 1]) + (tile[5][cy - 1][cx] - tile[5][cy + 1][cx]);
+            bout[k] = emf_update(c.w0, c.w1, w1k, cur[0], s[0], dx);
+            bout[k + n] = emf_update(c.w0, c.w1, w1k, cur[1], s[1], dy);
+            bout[k + 2 * n] = emf_update(c.w0, c.w1, w1k, cur[2], s[2], dz);
         }
         __syncthreads();
 #pragma unroll
@@ -507,12 +472,10 @@ __device__ __forceinline__ void march_tile(const Geo& g, const T* __restrict__ b
             cur[v] = nxt[v];
         }
         if (z + 1 < z1) {
-            if constexpr (EMF) {
-                T be[3];
-                bext_at(c.bext_z, c.be, za, be);
-                if constexpr (XY) bext_add_xy(c.bext_xy, P, p, be);
-                node_emf(ahd, be, c.sq);
-            }
+            T be[3];
+            bext_at(c.bext_z, c.be, za, be);
+            if constexpr (XY) bext_add_xy(c.bext_xy, P, p, be);
+            node_emf(ahd, be, c.sq);
 #pragma unroll
             for (int v = 0; v < 6; ++v) nxt[v] = ahd[v];
         }
@@ -725,9 +688,9 @@ __device__ __forceinline__ void ib_marker(const IBView<T>& ib, const T* __restri
     for (int j = 0; j < 9; ++j) {
         const T w = ib.mk_w[9 * m + j];
         const int q = base + ib.mk_q[9 * m + j];
-        a0 += w * f[q];
-        a1 += w * f[q + n];
-        a2 += w * f[q + 2 * n];
+        a0 = fma_rn(w, f[q], a0);
+        a1 = fma_rn(w, f[q + n], a1);
+        a2 = fma_rn(w, f[q + 2 * n], a2);
     }
     const T sm = ib.mk_s[m];
     ib.delta[3 * m + 0] = -sm * a0;
@@ -742,9 +705,9 @@ __device__ __forceinline__ void ib_shell(const IBView<T>& ib, T* __restrict__ f,
     for (int e = e0; e < e1; ++e) {
         const T w = ib.csr_w[e];
         const int m = ib.csr_mg[e];
-        c0 += w * ib.delta[3 * m + 0];
-        c1 += w * ib.delta[3 * m + 1];
-        c2 += w * ib.delta[3 * m + 2];
+        c0 = fma_rn(w, ib.delta[3 * m + 0], c0);
+        c1 = fma_rn(w, ib.delta[3 * m + 1], c1);
+        c2 = fma_rn(w, ib.delta[3 * m + 2], c2);
     }
     const int q = ib.shell_node[i];
     f[q] += c0;
@@ -876,9 +839,9 @@ __device__ __forceinline__ void ib_staged_plane(const IBView<T>& ib, T* f, int n
         for (int j = 0; j < 9; ++j) {
             const T w = tw[9 * m + j];
             const int q = tslot[9 * m + j];
-            a0 += w * sf[q];
-            a1 += w * sf[S + q];
-            a2 += w * sf[2 * S + q];
+            a0 = fma_rn(w, sf[q], a0);
+            a1 = fma_rn(w, sf[S + q], a1);
+            a2 = fma_rn(w, sf[2 * S + q], a2);
         }
         const T sm = tsc[m];
         sdelta[3 * m + 0] = -sm * a0;
@@ -910,9 +873,9 @@ __device__ __forceinline__ void ib_staged_plane(const IBView<T>& ib, T* f, int n
                     const int l[4] = {mm[u].x, mm[u].y, mm[u].z, mm[u].w};
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        c[u][0] += ww[u][e] * sdelta[3 * l[e] + 0];
-                        c[u][1] += ww[u][e] * sdelta[3 * l[e] + 1];
-                        c[u][2] += ww[u][e] * sdelta[3 * l[e] + 2];
+                        c[u][0] = fma_rn(ww[u][e], sdelta[3 * l[e] + 0], c[u][0]);
+                        c[u][1] = fma_rn(ww[u][e], sdelta[3 * l[e] + 1], c[u][1]);
+                        c[u][2] = fma_rn(ww[u][e], sdelta[3 * l[e] + 2], c[u][2]);
                     }
                 }
             }

@@ -8,6 +8,7 @@
 #include "qslbm_internal.h"
 #include "qslbm_kernels.cuh"
 #include "qslbm_resident.cuh"
+#include "qslbm_resident64.cuh"
 
 namespace qslbm {
 
@@ -308,10 +309,52 @@ struct Launch {
 
     static bool small_plane(const State& s) { return (long long)s.nx * s.ny <= (long long)kResidentSmallPlane; }
 
+    static auto resident64_kernel(const State& s) {
+        return s.nx * s.ny <= 4 * kRes64Threads ? k_sweeps_resident64<T, 4> : k_sweeps_resident64<T, kRes64MaxNpt>;
+    }
+
+    // FP64: one plane per CTA in 3-D, one thread-block cluster in 2-D.
+    static void launch_resident64(State& s, int nsweeps, const SweepCoef<T>& c, const IBView<T>& v,
+                                  cudaStream_t st) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.stream = st;
+        cfg.dynamicSmemBytes = s.resident_smem;
+        cudaLaunchAttribute attr[1];
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        const T* bin = (const T*)s.b[s.bcur];
+        T* bout = (T*)s.b[1 - s.bcur];
+        const T* u = (const T*)s.u[s.fcur];
+        cudaError_t e;
+        if (s.dim == 3) {
+            cfg.gridDim = dim3((unsigned)s.nz);
+            cfg.blockDim = dim3(kRes64Threads);
+            attr[0].id = cudaLaunchAttributeCooperative;
+            attr[0].val.cooperative = 1;
+            e = cudaLaunchKernelEx(&cfg, resident64_kernel(s), geo(s), bin, bout, u, c, v, (T*)s.xbuf,
+                                   (ResidentSync*)s.rsync, nsweeps, s.ib.max_ring, s.ib.max_shell, s.ib.max_nnz);
+        } else {
+            cfg.gridDim = dim3((unsigned)s.c2_ctas);
+            cfg.blockDim = dim3(kC2Threads);
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = (unsigned)s.c2_ctas;
+            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+            const C2Geo g{s.nx, s.ny, s.c2_rows, s.c2_mk, s.c2_sh, s.c2_nnz};
+            e = cudaLaunchKernelEx(&cfg, k_sweeps_cluster64<T>, g, bin, bout, u, c, v, nsweeps);
+        }
+        if (e != cudaSuccess) s.launch_error = true;
+    }
+
     static void launch_resident(State& s, int nsweeps, const SweepCoef<T>& c, const IBView<T>& v,
                                 cudaStream_t st) {
+        if constexpr (sizeof(T) == 8) {
+            if (s.dim == 3 || s.c2_ctas > 0) {
+                launch_resident64(s, nsweeps, c, v, st);
+                return;
+            }
+        }
         const bool small = small_plane(s);
-        if (s.dim == 3) {
+        if constexpr (sizeof(T) == 4) if (s.dim == 3) {
             if (s.resident_uhalo) {
                 if (small)
                     resident_launch_one<3, true, true>(s, nsweeps, c, v, st);
@@ -323,12 +366,12 @@ struct Launch {
                 else
                     resident_launch_one<3, false, false>(s, nsweeps, c, v, st);
             }
-        } else {
-            if (small)
-                resident_launch_one<2, false, true>(s, nsweeps, c, v, st);
-            else
-                resident_launch_one<2, false, false>(s, nsweeps, c, v, st);
+            return;
         }
+        if (small)
+            resident_launch_one<2, false, true>(s, nsweeps, c, v, st);
+        else
+            resident_launch_one<2, false, false>(s, nsweeps, c, v, st);
     }
 
     template <int DIM, bool UHALO, bool SMALL>
@@ -415,6 +458,89 @@ struct Launch {
         return cudaSuccess;
     }
 
+    // FP64, 3-D: shared memory for b, e and the IB tables, every plane's CTA
+    // co-resident.
+    static cudaError_t try_resident64(State& s, size_t smem, int sms, bool& ok) {
+        ok = false;
+        if ((long long)s.nx * s.ny > (long long)kRes64Threads * kRes64MaxNpt) return cudaSuccess;
+        const auto kern = resident64_kernel(s);
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+            cudaSuccess) {
+            cudaGetLastError();
+            return cudaSuccess;
+        }
+        int per_sm = 0;
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kRes64Threads, smem);
+        if (e != cudaSuccess) return e;
+        ok = per_sm >= 1 && (long long)per_sm * sms >= s.nz;
+        return cudaSuccess;
+    }
+
+    // FP64, 2-D: the plane's rows over the CTAs of one cluster, the largest
+    // cluster (at most 16) that the device can hold with a row or more per
+    // CTA: one SM does about two FP64 operations per clock, so the sweep time
+    // falls nearly with the CTA count.
+    static cudaError_t plan_cluster2d(State& s, int optin) {
+        s.c2_ctas = 0;
+        const HostIB& h = s.hib;
+        const int R = s.ib.max_ring, S = s.ib.max_shell;
+        for (int C = kC2MaxCluster; C >= 1; C /= 2) {
+            if (C > s.ny) continue;
+            const int RB = (s.ny + C - 1) / C;
+            int mk = 1, sh = 1, nnz = 1;
+            for (int r = 0; r * RB < s.ny; ++r) {
+                const int y0 = r * RB, y1 = std::min(y0 + RB, s.ny);
+                int m = 0, k = 0, e = 0;
+                for (int j = 0; j < R; ++j) {
+                    bool own = false;
+                    for (int b = 0; b < 3; ++b) own = own || (h.iy[3 * j + b] >= y0 && h.iy[3 * j + b] < y1);
+                    m += own;
+                }
+                for (int i = 0; i < S; ++i) {
+                    const int y = h.shell_xy[i] / s.nx;
+                    if (y >= y0 && y < y1) {
+                        ++k;
+                        e += h.csr_off[i + 1] - h.csr_off[i];
+                    }
+                }
+                mk = std::max(mk, m);
+                sh = std::max(sh, k);
+                nnz = std::max(nnz, e);
+            }
+            const size_t smem = cluster2d_smem_bytes(s.nx, RB, R, mk, sh, nnz);
+            if (smem + 1024 > (size_t)optin) continue;
+            cudaError_t e = cudaSuccess;
+            if (C > 8) e = cudaFuncSetAttribute(k_sweeps_cluster64<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(k_sweeps_cluster64<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)C);
+            cfg.blockDim = dim3(kC2Threads);
+            cfg.dynamicSmemBytes = smem;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = (unsigned)C;
+            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            int clusters = 0;
+            if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, k_sweeps_cluster64<T>, &cfg);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                continue;
+            }
+            if (clusters < 1) continue;
+            s.c2_ctas = C;
+            s.c2_rows = RB;
+            s.c2_mk = mk;
+            s.c2_sh = sh;
+            s.c2_nnz = nnz;
+            s.resident_smem = smem;
+            return cudaSuccess;
+        }
+        return cudaSuccess;
+    }
+
     static cudaError_t plan_resident(State& s) {
         s.resident = false;
         const long long P = (long long)s.nx * s.ny;
@@ -429,8 +555,24 @@ struct Launch {
         const size_t halo = (size_t)6 * P * sizeof(T);
         const size_t reserve = 1024;  // static shared variables and the runtime's own share
         bool ok = false;
-        if (s.dim == 3 && base + halo + reserve <= (size_t)optin) {
-            if ((e = try_resident<3, true>(s, base + halo, ok)) != cudaSuccess) return e;
+        if constexpr (sizeof(T) == 8) {
+            if (s.dim == 2) {
+                if ((e = plan_cluster2d(s, optin)) != cudaSuccess) return e;
+                s.resident = s.c2_ctas > 0;
+                if (s.resident) return cudaSuccess;
+            } else {
+                int sms = 0;
+                if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+                if (base + reserve > (size_t)optin) return cudaSuccess;
+                if ((e = try_resident64(s, base, sms, ok)) != cudaSuccess) return e;
+                s.resident = ok;
+                s.resident_smem = base;
+                return cudaSuccess;
+            }
+        }
+        if (sizeof(T) == 4 && s.dim == 3 && base + halo + reserve <= (size_t)optin) {
+            if constexpr (sizeof(T) == 4)
+                if ((e = try_resident<3, true>(s, base + halo, ok)) != cudaSuccess) return e;
             if (ok) {
                 s.resident = true;
                 s.resident_uhalo = true;
@@ -439,10 +581,10 @@ struct Launch {
             }
         }
         if (base + reserve > (size_t)optin) return cudaSuccess;
-        if (s.dim == 3)
-            e = try_resident<3, false>(s, base, ok);
-        else
+        if (s.dim == 2)
             e = try_resident<2, false>(s, base, ok);
+        else if constexpr (sizeof(T) == 4)
+            e = try_resident<3, false>(s, base, ok);
         if (e != cudaSuccess) return e;
         if (ok) {
             s.resident = true;
