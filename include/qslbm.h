@@ -75,8 +75,9 @@ extern "C" {
  * memory (the band's rows are staged by the tensor memory accelerator with
  * three halo rows on each side); FP32, 3-D, nx a multiple of 4 up to 256, the
  * same wall ring on every plane; create fails with QSLBM_EINVAL otherwise.
- * AUTO picks RESIDENT when it fits; else, when FUSED applies, it times FUSED
- * and SPLIT on the handle's fields at creation (without changing them) and
+ * AUTO picks RESIDENT when it fits (in FP32 also with several planes per CTA and
+ * with an in-plane field, forms that a request for RESIDENT by name does not
+ * take); else, when FUSED applies, it times FUSED and SPLIT on the handle's fields at creation (without changing them) and
  * keeps FUSED only when it is at least 2 % faster (the two give bitwise equal
  * results); else SPLIT. */
 /* Initial velocity: rest (plus the seeded noise), or the Ha = 0 profile

@@ -756,11 +756,15 @@ int create_impl(const qslbm_params* pin, qslbm_handle** out) {
         }
     }
     if (s.resident) {
-        const size_t xb = (size_t)2 * (s.esz == 8 ? 5 : 3) * s.n * s.esz;
+        // plane exchange: values of every plane, or the slab kernel's messages
+        s.xbuf_bytes = s.slab_ctas > 0 ? s.slab_xbytes
+                                       : (size_t)2 * (s.esz == 8 ? 5 : 3) * s.n * s.esz;
         const size_t sb = sizeof(unsigned int) * (4 + (size_t)s.nz);
-        if ((rc = dev_alloc(s, &s.xbuf, xb))) goto fail;
+        if ((rc = dev_alloc(s, &s.xbuf, s.xbuf_bytes))) goto fail;
         if ((rc = dev_alloc(s, &s.rsync, sb))) goto fail;
+        if (s.slab_ctas > 0 && s.slab_rows > 3 && (rc = dev_alloc(s, (void**)&s.slab_S, 3 * fb))) goto fail;
         cudaError_t e = cudaMemsetAsync(s.rsync, 0, sb, s.stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(s.xbuf, 0, s.xbuf_bytes, s.stream);
         if (e != cudaSuccess) {
             rc = cuda_fail(e, "cudaMemsetAsync");
             goto fail;
@@ -903,6 +907,7 @@ int check_resident(State& s) {
     QCHK(cudaStreamSynchronize(s.stream));
     if (!err) return QSLBM_OK;
     QCHK(cudaMemsetAsync(s.rsync, 0, sizeof(unsigned int) * (4 + (size_t)s.nz), s.stream));
+    QCHK(cudaMemsetAsync(s.xbuf, 0, s.xbuf_bytes, s.stream));
     QCHK(cudaStreamSynchronize(s.stream));
     g_last_error = "resident sweep kernel: neighbour wait timed out";
     return QSLBM_ETIMEOUT;

@@ -104,6 +104,11 @@ struct State {
     int ib_staged_u = 1;        // its shell nodes per thread per batch of loads (1, 2 or 5)
     bool resident_uhalo = false;
     size_t resident_smem = 0;
+    // FP32 slab kernel: CTAs (0: not used), rows per thread, threads, list entries
+    // past each shell node's fourth
+    int slab_ctas = 0, slab_rows = 0, slab_threads = 0, slab_more = 0;
+    size_t xbuf_bytes = 0, slab_xbytes = 0;  // exchange of the resident kernels; the slab kernel's
+    float* slab_S = nullptr;           // [3][n] the applied field's share, when it does not fit on chip
     // FP64 2-D resident kernel: CTAs of its cluster (0: not used), rows per CTA,
     // largest band's markers, shell nodes and list entries
     int c2_ctas = 0, c2_rows = 0, c2_mk = 0, c2_sh = 0, c2_nnz = 0;
@@ -160,7 +165,8 @@ struct Ops {
     void (*to_f64)(State&, cudaStream_t);               // staging <- state
     void (*from_f64)(State&, int mask, cudaStream_t);   // state <- staging
     // decide whether the resident sweep kernel fits this domain; sets
-    // s.resident, s.resident_uhalo, s.resident_smem (no allocation)
+    // s.resident, s.resident_uhalo, s.resident_smem and the kernel's own shape
+    // (no allocation)
     cudaError_t (*plan_resident)(State&);
     cudaError_t (*plan_march)(State&);  // sets s.march_chunk and s.ib_staged_smem
     // launch shape of the fused sweep for the tables already in s (fu_TY,

@@ -9,6 +9,7 @@
 #include "qslbm_kernels.cuh"
 #include "qslbm_resident.cuh"
 #include "qslbm_resident64.cuh"
+#include "qslbm_slab.cuh"
 
 namespace qslbm {
 
@@ -309,6 +310,82 @@ struct Launch {
 
     static bool small_plane(const State& s) { return (long long)s.nx * s.ny <= (long long)kResidentSmallPlane; }
 
+    // FP32: a slab of planes per CTA
+    static auto slab_kernel(int K) {
+        return K == 1   ? k_sweeps_slab<1>
+               : K == 2 ? k_sweeps_slab<2>
+               : K == 3 ? k_sweeps_slab<3>
+               : K == 4 ? k_sweeps_slab<4>
+                        : k_sweeps_slab<5>;
+    }
+    static void launch_slab(State& s, int nsweeps, const SweepCoef<float>& c, const IBView<float>& v,
+                            cudaStream_t st) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)s.slab_ctas);
+        cfg.blockDim = dim3((unsigned)s.slab_threads);
+        cfg.dynamicSmemBytes = s.resident_smem;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        const cudaError_t e =
+            cudaLaunchKernelEx(&cfg, slab_kernel(s.slab_rows), geo(s), (const float*)s.b[s.bcur],
+                               (float*)s.b[1 - s.bcur], (const float*)s.u[s.fcur], c, v, s.slab_S, (float*)s.xbuf,
+                               (ResidentSync*)s.rsync, nsweeps, s.slab_more);
+        if (e != cudaSuccess) s.launch_error = true;
+    }
+
+    // The slab kernel for this domain: the fewest planes per CTA at which every
+    // CTA is co-resident.
+    static cudaError_t plan_slab(State& s, int optin, int sms) {
+        s.slab_ctas = 0;
+        if (s.dim != 3 || (long long)s.nx * s.ny > kResidentMaxPlane || !s.ib.zinv) return cudaSuccess;
+        const int ctas = (s.nz + (s.nz + sms - 1) / sms - 1) / ((s.nz + sms - 1) / sms);
+        const int G = (s.nz + ctas - 1) / ctas;  // the largest slab of the balanced split
+        const int K = slab_rows(s.nx, s.ny, G);
+        if (K == 0 || (long long)G * slab_plane_stride(s.nx, s.ny, G, K) > slab_half(K)) return cudaSuccess;
+        // Where it is not the faster one (measured, us per sweep, slab against the
+        // other): even-width planes of one per CTA beyond one row per thread stay
+        // with k_sweeps_resident (48x48: 5.3 against 5.0, 64x64: 7.1 against 7.05;
+        // at one row 24x24: 2.0 against 3.6, 36x36: 3.3 against 4.0), whose pairs an
+        // odd width does without (47x46: 5.3 against 6.8); even-width slabs of
+        // several planes at five rows stay with the marching sweep (60x60x304: 17.6
+        // against 16.6; at three rows 40x40x192: 7.5 against 9.5, at one row
+        // 24x24x300: 2.8 against 8.8).
+        if (s.nx % 2 == 0 && ((G == 1 && K > 1 && s.resident) || (G > 1 && K == kSlabMaxK))) return cudaSuccess;
+        // its start (tables, S) takes about 5 us longer than k_sweeps_resident's: a
+        // step of few sweeps does not earn that back
+        if (s.resident && s.units.n_mag < 24) return cudaSuccess;
+        const int R = s.ib.max_ring, S = s.ib.max_shell;
+        int more = 0;
+        for (int i = 0; i < S; ++i) more += std::max(0, s.hib.csr_off[i + 1] - s.hib.csr_off[i] - 4);
+        const size_t smem = slab_direct_smem_bytes(s.nx, s.ny, G, R, S, more);
+        if (smem + 1024 > (size_t)optin) return cudaSuccess;
+        const auto kern = slab_kernel(K);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return cudaSuccess;
+        }
+        int per_sm = 0;
+        // a thread per column of rows, and enough for a marker component or a
+        // shell node each
+        const int columns = G * slab_pairs(s.nx) * ((s.ny + K - 1) / K);
+        const int threads = std::min(kSlabThreads, (std::max(columns, std::max(3 * G * R, G * S)) + 31) / 32 * 32);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+        if (e != cudaSuccess) return e;
+        if ((long long)per_sm * sms < ctas) return cudaSuccess;
+        s.slab_ctas = ctas;
+        s.slab_rows = K;
+        s.slab_threads = threads;
+        s.slab_more = more;
+        s.slab_xbytes = (size_t)ctas * 4 * slab_msg_floats(s.nx, s.ny, G, K);
+        s.resident_smem = smem;
+        return cudaSuccess;
+    }
+
     static auto resident64_kernel(const State& s) {
         return s.nx * s.ny <= 4 * kRes64Threads ? k_sweeps_resident64<T, 4> : k_sweeps_resident64<T, kRes64MaxNpt>;
     }
@@ -350,6 +427,12 @@ struct Launch {
         if constexpr (sizeof(T) == 8) {
             if (s.dim == 3 || s.c2_ctas > 0) {
                 launch_resident64(s, nsweeps, c, v, st);
+                return;
+            }
+        }
+        if constexpr (sizeof(T) == 4) {
+            if (s.slab_ctas > 0) {
+                launch_slab(s, nsweeps, c, v, st);
                 return;
             }
         }
@@ -541,7 +624,27 @@ struct Launch {
         return cudaSuccess;
     }
 
+    // FP32, 3-D: the slab kernel wherever it fits.  A handle that asks for the
+    // resident kernel by name gets it where one plane per CTA fits the device
+    // (and no in-plane field is applied), as before the slab kernel.
     static cudaError_t plan_resident(State& s) {
+        const cudaError_t e = plan_planes(s);
+        if constexpr (sizeof(T) == 4) {
+            if (e != cudaSuccess || (!s.resident && s.p.sweep_kernel == QSLBM_SWEEP_RESIDENT)) return e;
+            int dev = 0, optin = 0, sms = 0;
+            cudaError_t f = cudaGetDevice(&dev);
+            if (f == cudaSuccess) f = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+            if (f == cudaSuccess) f = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            if (f == cudaSuccess) f = plan_slab(s, optin, sms);
+            if (s.slab_ctas > 0) s.resident = true;
+            return f;
+        }
+        return e;
+    }
+
+    // One plane per CTA (k_sweeps_resident, k_sweeps_resident64) or, in FP64
+    // and 2-D, one cluster.
+    static cudaError_t plan_planes(State& s) {
         s.resident = false;
         const long long P = (long long)s.nx * s.ny;
         if (P > (long long)kResidentMaxPlane) return cudaSuccess;
