@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(kNodeThreads, (kIbStagedMinBlocks<T, U>)) k_ba
     const InstDesc<T>& D = d[i];
     const int z = blockIdx.x - pfirst[i];
     T* f = D.b[((D.bpar + s) & 1) ^ 1];
-    ib_staged_plane<T, kNodeThreads, U>(D.ibm, f, (int)D.g.n, z * D.g.nx * D.g.ny, D.ibm.zinv ? 0 : z, max_ring,
+    ib_staged_plane<T, kNodeThreads, U, false>(D.ibm, f, (int)D.g.n, z * D.g.nx * D.g.ny, D.ibm.zinv ? 0 : z, max_ring,
                                      max_shell, smem_raw);
 }
 

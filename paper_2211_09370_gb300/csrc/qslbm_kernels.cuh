@@ -491,189 +491,290 @@ __global__ void __launch_bounds__(kMarchTX* kMarchTY) k_sweep_march(Geo g, const
     march_tile<T, XY>(g, bin, bout, u, c, blockIdx.x, blockIdx.y, blockIdx.z, chunk, tile);
 }
 
-// FP32 z-marching sweep on x-adjacent node pairs (nx even): a CTA of 256
-// threads owns a tile of kPairTXP pairs (32 nodes) x kPairTY rows and walks a
-// chunk of z planes; every global access moves two nodes (8 bytes), so the
-// address arithmetic, loads, stores and loop overhead per node are half those
-// of march_tile.  EMF form as in march_tile.  The staged plane is
+// FP32 z-marching sweep on x-adjacent node pairs: a CTA of 128 threads owns a
+// tile of 32 x 16 nodes and walks a chunk of z planes; a thread owns a node pair
+// in each of two rows.  EMF form as in march_tile, in packed arithmetic (one
+// instruction for a pair, the same roundings).  The staged plane is
 // double-buffered (one barrier per plane) and every global load is issued one
-// plane ahead of its use: the column's plane z + 2, the halo's plane z + 1.
+// plane ahead of its use: the columns' plane z + 2, the halo's plane z + 1.  The
+// tile is the same for every plane: shapes chosen to leave fewer idle threads
+// (such as 44 columns for a width of 88) lost more to unaligned rows and index
+// arithmetic (88x88x300 32.9 us against 26.7).
+//
+// What bounds it on domains above L2 is memory bandwidth, once shared-memory
+// wavefronts and instruction issue are out of the way: two rows per thread halve
+// the y neighbours read from shared memory, and a component's even and odd
+// columns lie apart, so that a warp's accesses to either node of its pairs and to
+// their x neighbours are consecutive words (stored side by side, every x
+// neighbour was a two-way bank conflict).  An even width moves a pair as one
+// 8-byte access; an odd one, whose rows start at odd nodes, as two.  Sweep alone,
+// 96x96x512: 37.2 us against 40.0 with one row per thread and scalar arithmetic
+// (4.6 TB/s of the 36 B a node; 15.8 M warp instructions against 21.4 M), with the
+// IB 49.3 against 51.0; 72x72x384 27.2 against 30.7; 89x89x300 (one scalar node
+// per thread before) 31.7 against 36.5.  (L2 eviction hints on u, b or the new b:
+// 39.8 to 44 us at 96x96x512.)  The batch keeps march_tile: its small members
+// leave most of a 32 x 16 tile idle (12 pipes of 40^2 to 58^2 44.9 ms against 40.1).
 constexpr int kPairTXP = 16, kPairTY = 16;
-constexpr int kPairThreads = kPairTXP * kPairTY;
-// tile row: pad, left halo, 32 nodes, right halo, pad (pairs start at even columns)
-constexpr int kPairW = 2 * kPairTXP + 4;
-using PairTile = float[2][6][kPairTY + 2][kPairW];
+constexpr int kPairThreads = kPairTXP * kPairTY / 2;
+// Floats between two rows of a staged half: a warp covers two thread rows, two
+// tile rows apart, whose 16 columns have to lie 16 banks apart (17, unpadded, puts
+// them 2 banks apart).
+constexpr int kPairRow = 24;
+// Floats of one half (even or odd columns) of a field in the staged tile.
+constexpr int kPairHalf = (kPairTY + 2) * kPairRow;
+static_assert(2 * kPairTXP + 2 * kPairTY <= kPairThreads, "one halo item a thread");
+// [buffer][field][even, odd][row][column]; rows: the tile's and one halo row on
+// each side; even column c is node 2c (one past the last: the halo right of the
+// tile), odd column c is node 2c - 1 (0: the halo left of it)
+using PairTile = float[2][6][2][kPairHalf];
 
-// Halo item hid of a pair tile (64 items): 0-15 the pairs of the row above,
-// 16-31 the row below, 32-47 the column left of the tile, 48-63 the column
-// right of it (corners are not needed by the 5-point in-plane stencil).
-// kind: 0 none, 1 pair, 2 single node; gp: in-plane index (periodic image).
-__device__ __forceinline__ void pair_halo(int hid, int x0, int y0, int nx, int ny, int& kind, int& row, int& col,
-                                          int& gp) {
+// Halo item hid of a pair tile: the pairs of the row above, of the row below, the
+// nodes of the column left of the tile, of the column right of it (corners are not
+// needed by the 5-point in-plane stencil).  kind: 0 none, 1 pair, 2 left node,
+// 3 right node; at: its offset in a staged half; gp, gq: in-plane indices of its
+// nodes (periodic images).
+__device__ __forceinline__ void pair_halo(int hid, int x0, int y0, int nx, int ny, int& kind, int& at, int& gp,
+                                          int& gq) {
     kind = 0;
-    row = 0;
-    col = 0;
-    gp = 0;
-    if (hid >= 64) return;
-    int gx, gy;
-    if (hid < 32) {
-        const int j = hid & 15;
+    at = 0;
+    gp = gq = 0;
+    if (hid >= 2 * kPairTXP + 2 * kPairTY) return;
+    if (hid < 2 * kPairTXP) {
+        const bool above = hid < kPairTXP;
+        const int col = above ? hid : hid - kPairTXP;
         kind = 1;
-        row = hid < 16 ? 0 : kPairTY + 1;
-        col = 2 + 2 * j;
-        gx = (x0 + 2 * j) % nx;
-        gy = hid < 16 ? (y0 - 1 + ny) % ny : (y0 + kPairTY) % ny;
+        at = (above ? 0 : kPairTY + 1) * kPairRow + col;
+        const int gx = (x0 + 2 * col) % nx, gy = above ? (y0 - 1 + ny) % ny : (y0 + kPairTY) % ny;
+        gp = gy * nx + gx;
+        gq = gy * nx + (gx + 1) % nx;
     } else {
-        const int i = hid & 15;
-        kind = 2;
-        row = 1 + i;
-        col = hid < 48 ? 1 : 2 * kPairTXP + 2;
-        gx = hid < 48 ? (x0 - 1 + nx) % nx : (x0 + 2 * kPairTXP) % nx;
-        gy = (y0 + i) % ny;
+        const int j = hid - 2 * kPairTXP;
+        const bool left = j < kPairTY;
+        const int i = left ? j : j - kPairTY;
+        kind = left ? 2 : 3;
+        at = (1 + i) * kPairRow + (left ? 0 : kPairTXP);
+        const int gx = left ? (x0 - 1 + nx) % nx : (x0 + 2 * kPairTXP) % nx;
+        gp = gq = ((y0 + i) % ny) * nx + gx;
     }
-    gp = gy * nx + gx;
 }
 
+// Packed FP32 arithmetic on a node pair; sub2 rounds as a subtraction does.
+__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.f, -1.f), a); }  // a - b
+
+// node_emf of the two nodes of a pair; be: B^ext per component of both.
+__device__ __forceinline__ void pair_emf(float2 r[6], const float2 be[3], float sq) {
+    const float2 q = f2(sq, sq);
+    const float2 B0 = fma2(q, r[0], be[0]), B1 = fma2(q, r[1], be[1]), B2 = fma2(q, r[2], be[2]);
+    const float2 u0 = r[3], u1 = r[4], u2 = r[5];
+    const float2 t1 = mul2(u1, B0), t2 = mul2(u2, B0), t3 = mul2(u2, B1);
+    r[3] = fma2(u0, B1, f2(-t1.x, -t1.y));
+    r[4] = fma2(u0, B2, f2(-t2.x, -t2.y));
+    r[5] = fma2(u1, B2, f2(-t3.x, -t3.y));
+}
 __device__ __forceinline__ void pair_emf(float2 r[6], const float beA[3], const float beB[3], float sq) {
-    float a[6] = {r[0].x, r[1].x, r[2].x, r[3].x, r[4].x, r[5].x};
-    float b[6] = {r[0].y, r[1].y, r[2].y, r[3].y, r[4].y, r[5].y};
-    node_emf(a, beA, sq);
-    node_emf(b, beB, sq);
-#pragma unroll
-    for (int v = 0; v < 6; ++v) r[v] = make_float2(a[v], b[v]);
+    const float2 be[3] = {f2(beA[0], beB[0]), f2(beA[1], beB[1]), f2(beA[2], beB[2])};
+    pair_emf(r, be, sq);
 }
 
-template <typename F, bool XY>
-__global__ void __launch_bounds__(kPairThreads) k_sweep_march_pair(Geo g, const F* __restrict__ bin,
-                                                                   F* __restrict__ bout, const F* __restrict__ u,
-                                                                   SweepCoef<F> c, int chunk) {
-    static_assert(sizeof(F) == 4, "the pair sweep is the FP32 path");
-    __shared__ __align__(16) PairTile tile;
+// emf_update of a pair, and its in-plane and z sums: s of one component and the
+// flux difference d (march_tile's expressions in its order).
+__device__ __forceinline__ float2 pair_update(float w0, float w1, float w1k, float2 b, float2 s, float2 d) {
+    return fma2(f2(w0, w0), b, fma2(f2(w1k, w1k), d, mul2(f2(w1, w1), s)));
+}
+
+template <bool XY>
+__device__ __forceinline__ void pair_tile(const Geo& g, const float* __restrict__ bin, float* __restrict__ bout,
+                                          const float* __restrict__ u, const SweepCoef<float>& c, int bx, int by,
+                                          int bz, int chunk, PairTile& tile) {
     const int nx = g.nx, ny = g.ny, nz = g.nz;
     const int n = (int)g.n, P = nx * ny;
+    const bool even = (nx & 1) == 0;  // pairs lie on 8-byte boundaries
     const int tx = threadIdx.x % kPairTXP, ty = threadIdx.x / kPairTXP;
-    const int x0 = blockIdx.x * 2 * kPairTXP, y0 = blockIdx.y * kPairTY;
-    const int x = x0 + 2 * tx, y = y0 + ty;
-    const bool active = x < nx && y < ny;
-    const int p = (y % ny) * nx + (x % nx);  // even: a pair never straddles a row end
-    const int z0 = blockIdx.z * chunk;
+    const int x0 = bx * 2 * kPairTXP, y0 = by * kPairTY;
+    const int x = x0 + 2 * tx, y = y0 + 2 * ty;
+    const bool active[2] = {x < nx && y < ny, x < nx && y + 1 < ny};
+    // rows and columns past the domain's end stage the periodic images their
+    // neighbours need; p: the pairs' first nodes, dq: from there to the second
+    const int p[2] = {(y % ny) * nx + (x % nx), ((y + 1) % ny) * nx + (x % nx)};
+    const int dq = x % nx == nx - 1 ? 1 - nx : 1;
+    const bool two = x + 1 < nx;  // the second node is in the domain
+    const int z0 = bz * chunk;
     const int z1 = min(z0 + chunk, nz);
-    const float* src[6] = {bin, bin + n, bin + 2 * n, u, u + n, u + 2 * n};
-    int hkind, hrow, hcol, hp;
-    pair_halo(threadIdx.x, x0, y0, nx, ny, hkind, hrow, hcol, hp);
-    auto ld2 = [](const float* q) { return *reinterpret_cast<const float2*>(q); };
+    int hkind, hat, hp, hq;
+    pair_halo(threadIdx.x, x0, y0, nx, ny, hkind, hat, hp, hq);
+    // nodes k and k + d
+    auto load = [&](int k, int d, float2 r[6]) {
+        if (even) {
+#pragma unroll
+            for (int v = 0; v < 3; ++v) {
+                r[v] = *reinterpret_cast<const float2*>(bin + v * n + k);
+                r[3 + v] = *reinterpret_cast<const float2*>(u + v * n + k);
+            }
+        } else {
+#pragma unroll
+            for (int v = 0; v < 3; ++v) {
+                r[v] = f2(bin[v * n + k], bin[v * n + k + d]);
+                r[3 + v] = f2(u[v * n + k], u[v * n + k + d]);
+            }
+        }
+    };
     // halo values of plane zz (raw), pair or single node (in .x)
     auto load_halo = [&](int zz, float2 h[6]) {
         if (hkind == 1) {
+            load(zz * P + hp, hq - hp, h);
+        } else if (hkind != 0) {
+            const int k = zz * P + hp;
 #pragma unroll
-            for (int v = 0; v < 6; ++v) h[v] = ld2(src[v] + zz * P + hp);
-        } else if (hkind == 2) {
-#pragma unroll
-            for (int v = 0; v < 6; ++v) h[v] = make_float2(src[v][zz * P + hp], 0.f);
+            for (int v = 0; v < 3; ++v) {
+                h[v] = f2(bin[v * n + k], 0.f);
+                h[3 + v] = f2(u[v * n + k], 0.f);
+            }
         }
     };
-    // (b, u) -> (b, e) of the nodes pp and pp + 1 of plane zz
-    auto emf2 = [&](float2 r[6], int zz, int pp) {
+    // (b, u) -> (b, e) of the nodes pp and pp + d of plane zz
+    auto emf2 = [&](float2 r[6], int zz, int pp, int d) {
         float be[3];
         bext_at(c.bext_z, c.be, zz, be);
         if constexpr (XY) {
             float bA[3] = {be[0], be[1], be[2]}, bB[3] = {be[0], be[1], be[2]};
             bext_add_xy(c.bext_xy, P, pp, bA);
-            bext_add_xy(c.bext_xy, P, pp + 1 < P ? pp + 1 : pp, bB);
+            bext_add_xy(c.bext_xy, P, pp + d, bB);
             pair_emf(r, bA, bB, c.sq);
         } else {
             pair_emf(r, be, be, c.sq);
         }
     };
-    float2 prv[6], cur[6], nxt[6], ahd[6], hcur[6], hnxt[6];
+    float2 prv[2][6], cur[2][6], nxt[2][6], ahd[2][6], halo[6];
+    {
+        const int zm = wrap_dec(z0, nz), zn = wrap_inc(z0, nz);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            load(zm * P + p[r], dq, prv[r]);
+            load(z0 * P + p[r], dq, cur[r]);
+            load(zn * P + p[r], dq, nxt[r]);
+        }
+        load_halo(z0, halo);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            emf2(prv[r], zm, p[r], dq);
+            emf2(cur[r], z0, p[r], dq);
+            emf2(nxt[r], zn, p[r], dq);
+        }
+    }
+    const float w0 = c.w0, w1 = c.w1, w1k = c.w1 * c.kappa;
+    constexpr int rs = kPairRow;
+    const int at = (2 * ty + 1) * rs + tx;  // the pair's place in the halves
+    for (int z = z0; z < z1; ++z) {
+        const int zn = wrap_inc(z, nz);
+        const int za = wrap_inc(zn, nz);
+        auto& t = tile[z & 1];
+        float* const te = &t[0][0][at];  // fields 2 kPairHalf apart, the odd half kPairHalf on
+#pragma unroll
+        for (int v = 0; v < 6; ++v) {
+            te[2 * v * kPairHalf] = cur[0][v].x;
+            te[2 * v * kPairHalf + kPairHalf + 1] = cur[0][v].y;
+            te[2 * v * kPairHalf + rs] = cur[1][v].x;
+            te[2 * v * kPairHalf + kPairHalf + 1 + rs] = cur[1][v].y;
+        }
+        if (hkind != 0) {
+            emf2(halo, z, hp, hq - hp);  // a single halo node uses .x only
+            if (hkind == 1) {
+#pragma unroll
+                for (int v = 0; v < 6; ++v) {
+                    t[v][0][hat] = halo[v].x;
+                    t[v][1][hat + 1] = halo[v].y;
+                }
+            } else if (hkind == 2) {
+#pragma unroll
+                for (int v = 0; v < 6; ++v) t[v][1][hat] = halo[v].x;
+            } else {
+#pragma unroll
+                for (int v = 0; v < 6; ++v) t[v][0][hat] = halo[v].x;
+            }
+        }
+        if (z + 1 < z1) {
+#pragma unroll
+            for (int r = 0; r < 2; ++r) load(za * P + p[r], dq, ahd[r]);
+            load_halo(zn, halo);
+        }
+        __syncthreads();
+        // rows above and below the thread's two: b, e1, e3
+        float2 up[6], dn[6];
+        {
+            const float *tu = te - rs, *td = te + 2 * rs;
+#pragma unroll
+            for (int v = 0; v < 6; ++v)
+                if (v != 4) {
+                    up[v] = f2(tu[2 * v * kPairHalf], tu[2 * v * kPairHalf + kPairHalf + 1]);
+                    dn[v] = f2(td[2 * v * kPairHalf], td[2 * v * kPairHalf + kPairHalf + 1]);
+                }
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const float2* a_ = r == 0 ? up : cur[0];  // the row above
+            const float2* b_ = r == 0 ? cur[1] : dn;  // the row below
+            const float2* o = cur[r];
+            const float* tr = te + r * rs;
+            float lf[5], rt[5];  // x neighbours: b, e1, e2
+#pragma unroll
+            for (int v = 0; v < 5; ++v) {
+                lf[v] = tr[2 * v * kPairHalf + kPairHalf];
+                rt[v] = tr[2 * v * kPairHalf + 1];
+            }
+            const float2 d[3] = {
+                add2(sub2(b_[3], a_[3]), sub2(nxt[r][4], prv[r][4])),
+                add2(f2(lf[3] - o[3].y, o[3].x - rt[3]), sub2(nxt[r][5], prv[r][5])),
+                add2(f2(lf[4] - o[4].y, o[4].x - rt[4]), sub2(a_[5], b_[5]))};
+            if (active[r]) {
+                const int k = z * P + p[r];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const float2 s = add2(add2(f2(lf[a] + o[a].y, o[a].x + rt[a]), add2(a_[a], b_[a])),
+                                          add2(prv[r][a], nxt[r][a]));
+                    const float2 v = pair_update(w0, w1, w1k, o[a], s, d[a]);
+                    float* q = bout + k + a * n;
+                    if (even) {
+                        *reinterpret_cast<float2*>(q) = v;
+                    } else {
+                        q[0] = v.x;
+                        if (two) q[1] = v.y;
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int v = 0; v < 6; ++v) {
+                prv[r][v] = cur[r][v];
+                cur[r][v] = nxt[r][v];
+            }
+        if (z + 1 < z1) {
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                emf2(ahd[r], za, p[r], dq);
+#pragma unroll
+                for (int v = 0; v < 6; ++v) nxt[r][v] = ahd[r][v];
+            }
+        }
+    }
+}
+
+template <typename F, bool XY>
+__global__ void __launch_bounds__(kPairThreads, 3) k_sweep_march_pair(Geo g, const F* __restrict__ bin,
+                                                                      F* __restrict__ bout, const F* __restrict__ u,
+                                                                      SweepCoef<F> c, int chunk) {
+    static_assert(sizeof(F) == 4, "the pair sweep is the FP32 path");
+    __shared__ __align__(16) PairTile tile;
     // the IB pass after this sweep may be scheduled as this grid's CTAs exit;
     // b comes from the kernel before this one
     pdl_trigger();
     pdl_wait();
-    {
-        const int zm = wrap_dec(z0, nz), zn = wrap_inc(z0, nz);
-#pragma unroll
-        for (int v = 0; v < 6; ++v) {
-            prv[v] = ld2(src[v] + zm * P + p);
-            cur[v] = ld2(src[v] + z0 * P + p);
-            nxt[v] = ld2(src[v] + zn * P + p);
-        }
-        load_halo(z0, hcur);
-        emf2(prv, zm, p);
-        emf2(cur, z0, p);
-        emf2(nxt, zn, p);
-    }
-    const float w0 = c.w0, w1 = c.w1, w1k = c.w1 * c.kappa;
-    const int r = ty + 1, cc = 2 + 2 * tx;
-    for (int z = z0; z < z1; ++z) {
-        const int zn = wrap_inc(z, nz);
-        const int za = wrap_inc(zn, nz);
-        const int buf = z & 1;
-        if (z + 1 < z1) {
-#pragma unroll
-            for (int v = 0; v < 6; ++v) ahd[v] = ld2(src[v] + za * P + p);
-            load_halo(zn, hnxt);
-        }
-        auto& t = tile[buf];
-#pragma unroll
-        for (int v = 0; v < 6; ++v) *reinterpret_cast<float2*>(&t[v][r][cc]) = cur[v];
-        if (hkind != 0) {
-            emf2(hcur, z, hp);  // a single halo node uses .x only
-            if (hkind == 1) {
-#pragma unroll
-                for (int v = 0; v < 6; ++v) *reinterpret_cast<float2*>(&t[v][hrow][hcol]) = hcur[v];
-            } else {
-#pragma unroll
-                for (int v = 0; v < 6; ++v) t[v][hrow][hcol] = hcur[v].x;
-            }
-        }
-        __syncthreads();
-        if (active) {
-            float lf[6], rt[6];
-            float2 up[6], dn[6];
-#pragma unroll
-            for (int v = 0; v < 6; ++v) {
-                if (v != 5) {  // x neighbours: b, e1, e2
-                    lf[v] = t[v][r][cc - 1];
-                    rt[v] = t[v][r][cc + 2];
-                }
-                if (v != 4) {  // y neighbours: b, e1, e3
-                    up[v] = *reinterpret_cast<const float2*>(&t[v][r - 1][cc]);
-                    dn[v] = *reinterpret_cast<const float2*>(&t[v][r + 1][cc]);
-                }
-            }
-            const int k = z * P + p;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                const float sL = (lf[a] + cur[a].y) + (up[a].x + dn[a].x) + (prv[a].x + nxt[a].x);
-                const float sR = (cur[a].x + rt[a]) + (up[a].y + dn[a].y) + (prv[a].y + nxt[a].y);
-                float dL, dR;
-                if (a == 0) {
-                    dL = (dn[3].x - up[3].x) + (nxt[4].x - prv[4].x);
-                    dR = (dn[3].y - up[3].y) + (nxt[4].y - prv[4].y);
-                } else if (a == 1) {
-                    dL = (lf[3] - cur[3].y) + (nxt[5].x - prv[5].x);
-                    dR = (cur[3].x - rt[3]) + (nxt[5].y - prv[5].y);
-                } else {
-                    dL = (lf[4] - cur[4].y) + (up[5].x - dn[5].x);
-                    dR = (cur[4].x - rt[4]) + (up[5].y - dn[5].y);
-                }
-                *reinterpret_cast<float2*>(bout + k + a * n) =
-                    make_float2(emf_update(w0, w1, w1k, cur[a].x, sL, dL), emf_update(w0, w1, w1k, cur[a].y, sR, dR));
-            }
-        }
-#pragma unroll
-        for (int v = 0; v < 6; ++v) {
-            prv[v] = cur[v];
-            cur[v] = nxt[v];
-            hcur[v] = hnxt[v];
-        }
-        if (z + 1 < z1) {
-            emf2(ahd, za, p);
-#pragma unroll
-            for (int v = 0; v < 6; ++v) nxt[v] = ahd[v];
-        }
-    }
+    pair_tile<XY>(g, bin, bout, u, c, blockIdx.x, blockIdx.y, blockIdx.z, chunk, tile);
 }
 
 // Two-phase IB corrector over the whole domain (Sec. V.C-V.F): first one
@@ -782,7 +883,11 @@ __device__ __forceinline__ void ld4(const double* p, double (&w)[4]) {
 // the same order as ib_plane (the padding adds exact zeros).  tz: the plane
 // whose tables apply; smem as ib_staged_smem_bytes.  Called by every thread
 // of the CTA.
-template <typename T, int THREADS, int U>
+//
+// PRE: the places and lists of the thread's first U shell nodes are read before
+// the wait for the sweep too (36 registers at U = 4), so that only the shell
+// values' round trip follows it.
+template <typename T, int THREADS, int U, bool PRE>
 __device__ __forceinline__ void ib_staged_plane(const IBView<T>& ib, T* f, int n, int base, int tz, int max_ring,
                                                 int max_shell, unsigned char* smem) {
     const int m0 = ib.ring_off[tz], R = ib.ring_off[tz + 1] - m0;
@@ -804,14 +909,35 @@ __device__ __forceinline__ void ib_staged_plane(const IBView<T>& ib, T* f, int n
         tslot[e] = __ldg(ib.mk_slot + 9 * m0 + e);
     }
     for (int m = tid; m < R; m += THREADS) tsc[m] = __ldg(ib.mk_s + m0 + m);
-    pdl_wait();
-    for (int i0 = 0; i0 < S; i0 += U * THREADS) {
-        int q[U];
+    const int K = ib.pad_k;
+    int q[U];
+    int4 mm[U];
+    T ww[U][4];
+    auto lists = [&](int i0, int k0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * THREADS + tid;
+            if (i < S) {
+                const long long r = (long long)(s0 + i) * K + k0;
+                mm[u] = __ldg(reinterpret_cast<const int4*>(ib.pad_m + r));
+                ld4(ib.pad_w + r, ww[u]);
+            }
+        }
+    };
+    auto places = [&](int i0) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int i = i0 + u * THREADS + tid;
             q[u] = i < S ? __ldg(ib.shell_xy + s0 + i) : 0;
         }
+    };
+    if constexpr (PRE) {
+        places(0);
+        lists(0, 0);
+    }
+    pdl_wait();
+    for (int i0 = 0; i0 < S; i0 += U * THREADS) {
+        if (!PRE || i0 > 0) places(i0);
         T v[U][3];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -850,23 +976,12 @@ __device__ __forceinline__ void ib_staged_plane(const IBView<T>& ib, T* f, int n
     }
     __syncthreads();
     // (C) f += D^T delta on the shell, four list entries per load
-    const int K = ib.pad_k;
     for (int i0 = 0; i0 < S; i0 += U * THREADS) {
         T c[U][3];
 #pragma unroll
         for (int u = 0; u < U; ++u) c[u][0] = c[u][1] = c[u][2] = T(0);
         for (int k0 = 0; k0 < K; k0 += 4) {
-            int4 mm[U];
-            T ww[U][4];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int i = i0 + u * THREADS + tid;
-                if (i < S) {
-                    const long long r = (long long)(s0 + i) * K + k0;
-                    mm[u] = __ldg(reinterpret_cast<const int4*>(ib.pad_m + r));
-                    ld4(ib.pad_w + r, ww[u]);
-                }
-            }
+            if (!PRE || i0 > 0 || k0 > 0) lists(i0, k0);  // (PRE: the first four of the first U nodes are there)
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 if (i0 + u * THREADS + tid < S) {
@@ -880,14 +995,14 @@ __device__ __forceinline__ void ib_staged_plane(const IBView<T>& ib, T* f, int n
                 }
             }
         }
+        if (!PRE || S > U * THREADS) places(i0);  // (else as read before the wait)
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int i = i0 + u * THREADS + tid;
             if (i < S) {
-                const int q = __ldg(ib.shell_xy + s0 + i);
-                f0[q] = sf[i] + c[u][0];
-                f1[q] = sf[S + i] + c[u][1];
-                f2[q] = sf[2 * S + i] + c[u][2];
+                f0[q[u]] = sf[i] + c[u][0];
+                f1[q[u]] = sf[S + i] + c[u][1];
+                f2[q[u]] = sf[2 * S + i] + c[u][2];
             }
         }
     }
@@ -901,7 +1016,7 @@ __global__ void __launch_bounds__(kNodeThreads, (kIbStagedMinBlocks<T, U>))
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int z = blockIdx.x;
     pdl_trigger();  // the next sweep may be scheduled as these CTAs exit
-    ib_staged_plane<T, kNodeThreads, U>(ib, f, (int)g.n, z * g.nx * g.ny, ib.zinv ? 0 : z, max_ring, max_shell,
+    ib_staged_plane<T, kNodeThreads, U, (U == 2 || U == 4 || sizeof(T) == 8)>(ib, f, (int)g.n, z * g.nx * g.ny, ib.zinv ? 0 : z, max_ring, max_shell,
                                      smem_raw);
 }
 

@@ -112,22 +112,24 @@ struct Launch {
                 const T* u = (const T*)s.u[s.fcur];
                 if (pair_march(s)) {
                     const dim3 pgrid((unsigned)((s.nx + 2 * kPairTXP - 1) / (2 * kPairTXP)),
-                                     (unsigned)((s.ny + kPairTY - 1) / kPairTY), (unsigned)((s.nz + chunk - 1) / chunk));
+                                     (unsigned)((s.ny + kPairTY - 1) / kPairTY),
+                                     (unsigned)((s.nz + chunk - 1) / chunk));
                     if (s.bext_xy)
                         launch_pdl(k_sweep_march_pair<float, true>, pgrid, dim3(kPairThreads), 0, st, geo(s),
                                    (const float*)bin, (float*)bout, (const float*)u, fcoef(c), chunk);
                     else
                         launch_pdl(k_sweep_march_pair<float, false>, pgrid, dim3(kPairThreads), 0, st, geo(s),
                                    (const float*)bin, (float*)bout, (const float*)u, fcoef(c), chunk);
-                } else if (s.dim == 3)
-                {
-                    if (s.bext_xy)
-                        k_sweep_march<T, true><<<mgrid, kMarchTX * kMarchTY, 0, st>>>(geo(s), bin, bout, u, c, chunk);
-                    else
-                        k_sweep_march<T, false><<<mgrid, kMarchTX * kMarchTY, 0, st>>>(geo(s), bin, bout, u, c, chunk);
-                }
-                else
+                } else if (s.dim == 3) {
+                    if constexpr (sizeof(T) == 8) {
+                        if (s.bext_xy)
+                            k_sweep_march<T, true><<<mgrid, kMarchTX * kMarchTY, 0, st>>>(geo(s), bin, bout, u, c, chunk);
+                        else
+                            k_sweep_march<T, false><<<mgrid, kMarchTX * kMarchTY, 0, st>>>(geo(s), bin, bout, u, c, chunk);
+                    }
+                } else {
                     k_sweep_nodes<T, 2><<<grid, kNodeThreads, 0, st>>>(geo(s), bin, bout, u, c);
+                }
                 if (s.ib.nm > 0 && s.ib_staged_smem > 0) {
                     const int R = s.ib.max_ring, S = s.ib.max_shell;
                     const size_t sm = s.ib_staged_smem;
@@ -485,8 +487,8 @@ struct Launch {
         return try_resident_shape<DIM, UHALO, false>(s, smem, ok);
     }
 
-    // The FP32 pair kernel serves 3-D domains with an even nx.
-    static bool pair_march(const State& s) { return sizeof(T) == 4 && s.dim == 3 && s.nx % 2 == 0; }
+    // The pair kernel serves FP32 3-D domains.
+    static bool pair_march(const State& s) { return sizeof(T) == 4 && s.dim == 3; }
     static SweepCoef<float> fcoef(const SweepCoef<T>& c) {
         if constexpr (sizeof(T) == 4)
             return c;
@@ -500,19 +502,21 @@ struct Launch {
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const bool pair = pair_march(s);
-        if (e == cudaSuccess)
-            e = pair ? (s.bext_xy ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_march_pair<float, true>,
-                                                                                  kPairThreads, 0)
-                                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                                        &per_sm, k_sweep_march_pair<float, false>, kPairThreads, 0))
-                     : (s.bext_xy ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_march<T, true>,
-                                                                                  kMarchTX * kMarchTY, 0)
-                                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_march<T, false>,
-                                                                                  kMarchTX * kMarchTY, 0));
+        if (e == cudaSuccess) {
+            if constexpr (sizeof(T) == 4)
+                e = s.bext_xy ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_march_pair<T, true>,
+                                                                              kPairThreads, 0)
+                              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_march_pair<T, false>,
+                                                                              kPairThreads, 0);
+            else
+                e = s.bext_xy ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_march<T, true>,
+                                                                              kMarchTX * kMarchTY, 0)
+                              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_march<T, false>,
+                                                                              kMarchTX * kMarchTY, 0);
+        }
         if (e != cudaSuccess) return e;
-        const long long tiles =
-            pair ? (long long)((s.nx + 2 * kPairTXP - 1) / (2 * kPairTXP)) * ((s.ny + kPairTY - 1) / kPairTY)
-                 : (long long)((s.nx + kMarchTX - 1) / kMarchTX) * ((s.ny + kMarchTY - 1) / kMarchTY);
+        const int tx = pair ? 2 * kPairTXP : kMarchTX, ty = pair ? kPairTY : kMarchTY;
+        const long long tiles = (long long)((s.nx + tx - 1) / tx) * ((s.ny + ty - 1) / ty);
         const long long slots = (long long)std::max(1, per_sm) * std::max(1, sms);
         const long long per_column = std::max<long long>(1, slots / std::max<long long>(1, tiles));
         long long chunk = (s.nz + per_column - 1) / per_column;

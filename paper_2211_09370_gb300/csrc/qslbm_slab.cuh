@@ -133,12 +133,6 @@ __device__ __forceinline__ int slab_div(int t, int d, unsigned m) {
     return d > 1 ? (int)__umulhi((unsigned)t, m) : t;
 }
 
-__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.f, -1.f), a); }  // a - b
-
 __device__ __forceinline__ float2 slab_mul(float2 a, float2 b) { return mul2(a, b); }
 __device__ __forceinline__ float2 slab_sub(float2 a, float2 b) { return sub2(a, b); }
 __device__ __forceinline__ float2 slab_fma(float2 a, float2 b, float2 c) { return fma2(a, b, c); }
