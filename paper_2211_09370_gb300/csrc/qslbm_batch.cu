@@ -241,9 +241,10 @@ struct qslbm_batch {
     std::vector<qslbm::GroupDesc> h_groups;
     qslbm::GroupDesc* groups = nullptr;
     int groups_cap = 0;
-    float* xbuf = nullptr;               // exchange planes of every group
-    long long xbuf_cap = 0;              // floats
-    unsigned* gflags = nullptr;          // [groups_cap] sweep counters
+    uint4* xbuf = nullptr;               // messages of every group
+    long long xbuf_cap = 0, xbuf_used = 0;  // messages
+    int gstride = qslbm::kGroupStrideS;  // nodes a group holds, at most
+    unsigned* gcounts = nullptr;          // [groups_cap] sweeps done
     int* gerr = nullptr;                 // 1: a neighbour wait timed out
     int gcap = -1, goptin = 0;           // co-resident CTAs of the group kernel and its shared memory (bytes)
     cudaError_t launch_err = cudaSuccess;  // a launch of the group kernel that failed
@@ -387,6 +388,16 @@ void launch_sweep(qslbm_batch& B, int s, int threads, int grid, cudaStream_t st)
     }
 }
 
+// The group kernel for a shared-memory stride, with or without in-plane fields.
+auto group_kernel(int stride, bool xy) {
+    using D = qslbm::InstDesc<float>;
+    if (stride == qslbm::kGroupStrideL)
+        return xy ? qslbm::k_batch_resident<D, true, qslbm::kGroupStrideL>
+                  : qslbm::k_batch_resident<D, false, qslbm::kGroupStrideL>;
+    return xy ? qslbm::k_batch_resident<D, true, qslbm::kGroupStrideS>
+              : qslbm::k_batch_resident<D, false, qslbm::kGroupStrideS>;
+}
+
 // Every sweep of the resident groups' members: one cooperative launch (its
 // CTAs wait on one another, so all must be co-resident).
 template <typename T>
@@ -404,13 +415,8 @@ void launch_groups(qslbm_batch& B, cudaStream_t st) {
         attr[0].val.cooperative = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        cudaError_t e;
-        if (B.has_field)
-            e = cudaLaunchKernelEx(&cfg, qslbm::k_batch_resident<qslbm::InstDesc<float>, true>, d,
-                                   (const qslbm::GroupDesc*)B.groups, B.xbuf, B.gflags, B.gerr);
-        else
-            e = cudaLaunchKernelEx(&cfg, qslbm::k_batch_resident<qslbm::InstDesc<float>, false>, d,
-                                   (const qslbm::GroupDesc*)B.groups, B.xbuf, B.gflags, B.gerr);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, group_kernel(B.gstride, B.has_field), d,
+                                                 (const qslbm::GroupDesc*)B.groups, B.xbuf, B.gcounts, B.gerr);
         if (e != cudaSuccess) B.launch_err = e;
     }
 }
@@ -428,15 +434,16 @@ void launch_step(qslbm_batch& B, cudaStream_t st) {
 
 // Planes per group for a member that the resident group kernel can hold (0:
 // it cannot): FP32, a wall ring with the same tables on every plane, planes of
-// at most kGroupMaxNodes nodes, and a group's b, e and IB tables within the
-// opt-in shared memory.  The planes are split into the fewest groups, of
-// nearly equal size.
-int group_planes(const State& s, int optin) {
+// at most stride nodes, and a group's b, e and IB tables within the opt-in shared
+// memory.  The planes are split into the fewest groups, of nearly equal size.
+int group_planes(const State& s, int optin, int stride) {
     if (s.esz != 4 || s.dim != 3 || s.ib.nm == 0 || !s.ib.zinv || s.units.n_mag < 1) return 0;
     const int P = s.nx * s.ny;
-    if (P > qslbm::kGroupMaxNodes) return 0;
-    int G = std::min(s.nz, qslbm::kGroupMaxNodes / P);
-    while (G > 0 && qslbm::group_smem_bytes(s.ib.max_ring, s.ib.max_shell, s.ib.max_nnz, G) > (size_t)optin) --G;
+    if (P > stride) return 0;
+    int G = std::min(s.nz, stride / P);
+    while (G > 0 &&
+           qslbm::group_smem_bytes(stride, s.ib.max_ring, s.ib.max_shell, s.ib.max_nnz, G, P) > (size_t)optin)
+        --G;
     if (G == 0) return 0;
     const int ng = (s.nz + G - 1) / G;
     return (s.nz + ng - 1) / ng;  // the largest group of the balanced split
@@ -467,10 +474,10 @@ int build_groups(qslbm_batch& B) {
             g.prev = first + (j == 0 ? ng - 1 : j - 1);
             g.next = first + (j == ng - 1 ? 0 : j + 1);
             g.xoff = xoff;
-            xoff += 12LL * P;
+            xoff += qslbm::group_msgs(P);
             z0 += G;
             B.h_groups.push_back(g);
-            smem = std::max(smem, qslbm::group_smem_bytes(s.ib.max_ring, s.ib.max_shell, s.ib.max_nnz, G));
+            smem = std::max(smem, qslbm::group_smem_bytes(B.gstride, s.ib.max_ring, s.ib.max_shell, s.ib.max_nnz, G, P));
         }
     }
     B.ngroups = (int)B.h_groups.size();
@@ -478,31 +485,31 @@ int build_groups(qslbm_batch& B) {
     if (B.ngroups == 0) return QSLBM_OK;
     if (B.ngroups > B.groups_cap) {
         if (B.groups) cudaFree(B.groups);
-        if (B.gflags) cudaFree(B.gflags);
+        if (B.gcounts) cudaFree(B.gcounts);
         B.groups = nullptr;
-        B.gflags = nullptr;
+        B.gcounts = nullptr;
         const int cap = std::max(B.ngroups, 2 * B.groups_cap);
         BCHK(cudaMalloc((void**)&B.groups, sizeof(qslbm::GroupDesc) * cap));
-        BCHK(cudaMalloc((void**)&B.gflags, sizeof(unsigned) * cap));
+        BCHK(cudaMalloc((void**)&B.gcounts, sizeof(unsigned) * cap));
         B.groups_cap = cap;
     }
+    B.xbuf_used = xoff;
     if (xoff > B.xbuf_cap) {
         if (B.xbuf) cudaFree(B.xbuf);
         B.xbuf = nullptr;
         const long long cap = std::max(xoff, 2 * B.xbuf_cap);
-        BCHK(cudaMalloc((void**)&B.xbuf, sizeof(float) * cap));
+        BCHK(cudaMalloc((void**)&B.xbuf, sizeof(uint4) * cap));
         B.xbuf_cap = cap;
     }
     if (!B.gerr) BCHK(cudaMalloc((void**)&B.gerr, sizeof(int)));
     BCHK(cudaMemcpyAsync(B.groups, B.h_groups.data(), sizeof(qslbm::GroupDesc) * B.ngroups, cudaMemcpyHostToDevice,
                          B.stream));
-    BCHK(cudaMemsetAsync(B.gflags, 0, sizeof(unsigned) * B.ngroups, B.stream));
+    BCHK(cudaMemsetAsync(B.gcounts, 0, sizeof(unsigned) * B.ngroups, B.stream));
+    BCHK(cudaMemsetAsync(B.xbuf, 0, sizeof(uint4) * xoff, B.stream));
     BCHK(cudaMemsetAsync(B.gerr, 0, sizeof(int), B.stream));
-    for (bool xy : {false, true}) {
-        const void* fn = xy ? (const void*)qslbm::k_batch_resident<qslbm::InstDesc<float>, true>
-                            : (const void*)qslbm::k_batch_resident<qslbm::InstDesc<float>, false>;
-        BCHK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    }
+    for (bool xy : {false, true})
+        BCHK(cudaFuncSetAttribute((const void*)group_kernel(B.gstride, xy),
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     return QSLBM_OK;
 }
 
@@ -719,7 +726,8 @@ int check_groups(qslbm_batch& B) {
     BCHK(cudaMemcpyAsync(&bad, B.gerr, sizeof(int), cudaMemcpyDeviceToHost, B.stream));
     BCHK(cudaStreamSynchronize(B.stream));
     if (!bad) return QSLBM_OK;
-    BCHK(cudaMemsetAsync(B.gflags, 0, sizeof(unsigned) * B.ngroups, B.stream));
+    BCHK(cudaMemsetAsync(B.gcounts, 0, sizeof(unsigned) * B.ngroups, B.stream));
+    BCHK(cudaMemsetAsync(B.xbuf, 0, sizeof(uint4) * B.xbuf_used, B.stream));
     BCHK(cudaMemsetAsync(B.gerr, 0, sizeof(int), B.stream));
     BCHK(cudaStreamSynchronize(B.stream));
     qslbm::set_last_error("batched resident sweep: a neighbour wait timed out");
@@ -744,7 +752,7 @@ void destroy_batch(qslbm_batch* B) {
     if (B->graph_chunk) cudaGraphExecDestroy(B->graph_chunk);
     if (B->desc) cudaFree(B->desc);
     if (B->groups) cudaFree(B->groups);
-    if (B->gflags) cudaFree(B->gflags);
+    if (B->gcounts) cudaFree(B->gcounts);
     if (B->gerr) cudaFree(B->gerr);
     if (B->xbuf) cudaFree(B->xbuf);
     if (B->first) cudaFree(B->first);
@@ -766,7 +774,7 @@ int group_capacity(qslbm_batch& B) {
     BCHK(cudaGetDevice(&dev));
     BCHK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     BCHK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    const void* fn = (const void*)qslbm::k_batch_resident<qslbm::InstDesc<float>, true>;
+    const void* fn = (const void*)group_kernel(qslbm::kGroupStrideL, true);
     cudaFuncAttributes fa;
     BCHK(cudaFuncGetAttributes(&fa, fn));
     optin -= (int)fa.sharedSizeBytes;
@@ -811,24 +819,40 @@ int set_members(qslbm_batch* B, const std::vector<qslbm_handle*>& hs, const std:
         int rc0 = group_capacity(*B);
         if (rc0) return rc0;
         const int cap = B->gcap, optin = B->goptin;
-        std::vector<int> cand;
-        for (int i = 0; i < count; ++i) {
-            if (!allow.empty() && !allow[i]) continue;
-            gp[i] = group_planes(qslbm::handle_state_mut(hs[i]), optin);
-            if (gp[i] > 0) cand.push_back(i);
-        }
-        std::stable_sort(cand.begin(), cand.end(), [&](int a, int b) {
-            return qslbm::handle_state_mut(hs[a]).n < qslbm::handle_state_mut(hs[b]).n;
-        });
-        int used = 0;
         std::vector<int> adm;
-        for (int i : cand) {
-            const int ng = group_count(qslbm::handle_state_mut(hs[i]), gp[i]);
-            if (used + ng <= cap) {
-                used += ng;
-                adm.push_back(i);
-            } else {
-                gp[i] = 0;
+        long long held = -1;  // nodes of the admitted members
+        for (int stride : {qslbm::kGroupStrideS, qslbm::kGroupStrideL}) {
+            std::vector<int> g(count, 0), cand, a;
+            for (int i = 0; i < count; ++i) {
+                if (!allow.empty() && !allow[i]) continue;
+                g[i] = group_planes(qslbm::handle_state_mut(hs[i]), optin, stride);
+                if (g[i] > 0) cand.push_back(i);
+            }
+            std::stable_sort(cand.begin(), cand.end(), [&](int x, int y) {
+                return qslbm::handle_state_mut(hs[x]).n < qslbm::handle_state_mut(hs[y]).n;
+            });
+            int used = 0;
+            long long nodes = 0;
+            for (int i : cand) {
+                const State& s = qslbm::handle_state_mut(hs[i]);
+                const int ng = group_count(s, g[i]);
+                if (used + ng <= cap) {
+                    used += ng;
+                    nodes += s.n;
+                    a.push_back(i);
+                } else {
+                    g[i] = 0;
+                }
+            }
+            // the large stride where it holds more: a small member left to the
+            // marching sweep costs about as much per sweep as all the groups
+            // together (12 pipes of 24^2 to 28^2, 270 sweeps a step: a step of
+            // 2600 us against 4800 with eleven in groups and one marching)
+            if (nodes > held) {
+                held = nodes;
+                gp = g;
+                adm = a;
+                B->gstride = stride;
             }
         }
         // spread the admitted members over every co-resident CTA: the
@@ -843,7 +867,7 @@ int set_members(qslbm_batch* B, const std::vector<qslbm_handle*>& hs, const std:
             for (int i : adm) tot += group_count(qslbm::handle_state_mut(hs[i]), planes_at(i, T));
             return tot;
         };
-        int lo = 1, hi = qslbm::kGroupMaxNodes;  // groups_at(hi) <= cap
+        int lo = 1, hi = B->gstride;  // groups_at(hi) <= cap
         while (lo < hi) {
             const int mid = (lo + hi) / 2;
             if (groups_at(mid) <= cap)
@@ -983,7 +1007,7 @@ int qslbm_batch_info(const qslbm_batch* B, qslbm_batch_info_t* info) {
     info->sweep_grid = B->grid;
     long long nodes = 0, sweeps = 0;
     long long bytes = B->device_bytes + (long long)B->groups_cap * (sizeof(qslbm::GroupDesc) + sizeof(unsigned)) +
-                      B->xbuf_cap * (long long)sizeof(float) + (B->gerr ? (long long)sizeof(int) : 0);
+                      B->xbuf_cap * (long long)sizeof(uint4) + (B->gerr ? (long long)sizeof(int) : 0);
     for (qslbm_handle* h : B->members) {
         const State& s = qslbm::handle_state_mut(h);
         nodes += s.n;
@@ -1069,12 +1093,12 @@ double now_s(const qslbm_server& S) {
 
 // Groups of the resident group kernel a request would take at the largest
 // group size (-1: the kernel does not hold it: 2-D, no wall, planes above
-// kGroupMaxNodes nodes).
+// kGroupStrideS nodes).
 int groups_needed(const qslbm_params& p) {
     if (p.dim != 3 || p.geometry == QSLBM_PERIODIC) return -1;
     const long long P = (long long)p.nx * p.ny;
-    if (P > qslbm::kGroupMaxNodes || p.nz < 1) return -1;
-    const int G = std::max(1, std::min(p.nz, (int)(qslbm::kGroupMaxNodes / P)));
+    if (P > qslbm::kGroupStrideS || p.nz < 1) return -1;
+    const int G = std::max(1, std::min(p.nz, (int)(qslbm::kGroupStrideS / P)));
     return (p.nz + G - 1) / G;
 }
 

@@ -142,52 +142,6 @@ __device__ __forceinline__ float slab_fma(float a, float b, float c) { return __
 // c - a b
 __device__ __forceinline__ float2 nfma2(float2 a, float2 b, float2 c) { return __ffma2_rn(f2(-a.x, -a.y), b, c); }
 
-// A message: three values and a sequence number in two 64-bit words (a, hi16(b)
-// | seq) and (c, lo16(b) | seq), each of which carries the sequence's low 16
-// bits, so that a reader needs no order between the two words.
-struct Msg {
-    unsigned a, bs, c, bt;
-};
-__device__ __forceinline__ Msg msg_load(const uint4* p) {
-    unsigned long long lo, hi;
-    asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "l"(p) : "memory");
-    return Msg{(unsigned)lo, (unsigned)(lo >> 32), (unsigned)hi, (unsigned)(hi >> 32)};
-}
-// seq2: the sequence's low 16 bits twice
-__device__ __forceinline__ bool msg_stale(const Msg& m, unsigned seq2) { return __byte_perm(m.bs, m.bt, 0x5410) != seq2; }
-__device__ __forceinline__ void msg_values(const Msg& m, float& a, float& b, float& c) {
-    a = __uint_as_float(m.a);
-    b = __uint_as_float(__byte_perm(m.bs, m.bt, 0x3276));
-    c = __uint_as_float(m.c);
-}
-__device__ __forceinline__ void msg_store(bool go, uint4* p, float a, float b, float c, unsigned seq2) {
-    const unsigned f = __float_as_uint(b);
-    const unsigned bs = __byte_perm(f, seq2, 0x3254), bt = __byte_perm(f, seq2, 0x1054);
-    asm volatile(
-        "{\n\t.reg .pred q;\n\t.reg .b64 lo, hi;\n\t"
-        "setp.ne.u32 q, %5, 0;\n\t"
-        "mov.b64 lo, {%1, %2};\n\tmov.b64 hi, {%3, %4};\n\t"
-        "@q st.relaxed.gpu.global.v2.b64 [%0], {lo, hi};\n\t}" ::"l"(p),
-        "r"(__float_as_uint(a)), "r"(bs), "r"(__float_as_uint(c)), "r"(bt), "r"((unsigned)go)
-        : "memory");
-}
-__device__ __forceinline__ unsigned msg_seq2(unsigned seq) { return (seq & 0xffffu) * 0x10001u; }
-// After a poll that found a message stale (n: how many in a row, t0: the time of
-// the first look at the clock): true when the wait is to be given up, because a
-// second has passed or another thread of the CTA gave up, with the abort and
-// error flags raised.  The clock is read every 256 polls (a read takes longer
-// than a poll).
-__device__ __forceinline__ bool msg_give_up(unsigned& n, unsigned long long& t0, int* s_abort, int* err) {
-    if ((++n & 255u) != 0) return false;
-    const unsigned long long t = globaltimer_ns();
-    if (t0 == 0) t0 = t;
-    if (t - t0 > kWaitTimeoutNs) {
-        atomicExch(err, 1);
-        *(volatile int*)s_abort = 1;
-    }
-    return *(volatile int*)s_abort != 0;
-}
-
 // bytes (a multiple of 16) of shared memory to global memory, both 16-byte
 // aligned, by the bulk copy engine.
 __device__ __forceinline__ void slab_bulk_store(float* dst, const float* src, unsigned bytes) {
