@@ -8,7 +8,7 @@
 // and grid chosen by a timing autotuner when the batch is built.
 //
 // The per-node arithmetic is the single-instance code (march_tile, the IB sums
-// of ib_plane, force_node, flow_node), so a batched instance follows the same
+// of ib_plane, force_gather, flow_gather), so a batched instance follows the same
 // expressions as one stepped alone with the split sweep kernel.
 #include <cuda_runtime.h>
 
@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "qslbm.h"
+#include "qslbm_flow.cuh"
 #include "qslbm_groups.cuh"
 #include "qslbm_internal.h"
 #include "qslbm_kernels.cuh"
@@ -154,9 +155,9 @@ __global__ void __launch_bounds__(kNodeThreads) k_batch_force(const InstDesc<T>*
         const int y = p / nx;
         const int x = p - y * nx;
         if (D.flow_q == 27)  // uniform across the CTA (one instance plane)
-            force_node<T, 3, 27>(b, D.F, D.g.n, nx, ny, D.g.nz, x, y, z, (long long)z * P + p, D.fc, fb);
+            force_gather<T, 3, 27>(b, D.F, D.g.n, nx, ny, D.g.nz, x, y, z, D.fc, fb);
         else
-            force_node<T, 3>(b, D.F, D.g.n, nx, ny, D.g.nz, x, y, z, (long long)z * P + p, D.fc, fb);
+            force_gather<T, 3, 19>(b, D.F, D.g.n, nx, ny, D.g.nz, x, y, z, D.fc, fb);
     }
 }
 
@@ -174,13 +175,14 @@ __global__ void __launch_bounds__(kPlaneThreads) k_batch_flow(InstDesc<T>* __res
     const T* u = D.u[D.fpar];
     T* dro = D.drho[D.fpar ^ 1];
     T* uo = D.u[D.fpar ^ 1];
+    const FlowConst<T> c(D.flc);
     for (int p = threadIdx.x; p < P; p += blockDim.x) {
         const int y = p / nx;
         const int x = p - y * nx;
         if (D.flow_q == 27)
-            flow_node<T, 3, 27>(dr, u, D.F, dro, uo, n, nx, ny, nz, x, y, z, base + p, D.flc);
+            flow_gather<T, 3, 27>(dr, u, D.F, dro, uo, n, nx, ny, nz, x, y, z, base + p, c);
         else
-            flow_node<T, 3>(dr, u, D.F, dro, uo, n, nx, ny, nz, x, y, z, base + p, D.flc);
+            flow_gather<T, 3, 19>(dr, u, D.F, dro, uo, n, nx, ny, nz, x, y, z, base + p, c);
     }
     ib_plane<T>(D.ibu, uo, uo + n, uo + 2 * n, base, D.ibu.zinv ? 0 : z, sdelta);
     if (z == 0 && threadIdx.x == 0) *D.tdev += 1;

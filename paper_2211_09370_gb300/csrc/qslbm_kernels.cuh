@@ -1060,169 +1060,6 @@ __device__ __forceinline__ double flow_w(int j) {
 }
 
 // ---------------------------------------------------------------------------
-// Force: J = curl b by isotropic differences on the flow lattice
-// (d_beta phi = 3 sum_i w_i c_i,beta phi(x + c_i)), F = F_body(t) e_axis +
-// J x (B^ext + b).  One thread per node.
-template <typename T, int DIM, int Q = kDefaultFlowQ<DIM>>
-__device__ __forceinline__ void force_node(const T* __restrict__ b, T* __restrict__ F, long long n, int nx, int ny,
-                                           int nz, int x, int y, int z, long long k, const ForceCoef<T>& c,
-                                           T fb) {
-    const T* b1 = b + n;
-    const T* b2 = b + 2 * n;
-    T db[3][3];  // db[beta][alpha] = d_beta b_alpha
-#pragma unroll
-    for (int be = 0; be < 3; ++be)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) db[be][a] = T(0);
-#pragma unroll
-    for (int j = 1; j < Q; ++j) {
-        int cx, cy, cz;
-        flow_dir<Q>(j, cx, cy, cz);
-        const int q = (wrapi(z + cz, nz) * ny + wrapi(y + cy, ny)) * nx + wrapi(x + cx, nx);
-        const T w = (T)(3.0 * flow_w<Q>(j));
-        const T bq[3] = {b[q], b1[q], b2[q]};
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            if (cx) db[0][a] += (w * (T)cx) * bq[a];
-            if (cy) db[1][a] += (w * (T)cy) * bq[a];
-            if (cz) db[2][a] += (w * (T)cz) * bq[a];
-        }
-    }
-    const T J[3] = {db[1][2] - db[2][1], db[2][0] - db[0][2], db[0][1] - db[1][0]};
-    T Be[3];
-    bext_at(c.bext_z, c.be, z, Be);
-    bext_add_xy(c.bext_xy, nx * ny, y * nx + x, Be);
-    const T B[3] = {Be[0] + b[k], Be[1] + b[k + n], Be[2] + b[k + 2 * n]};
-    T L[3] = {J[1] * B[2] - J[2] * B[1], J[2] * B[0] - J[0] * B[2], J[0] * B[1] - J[1] * B[0]};
-    L[c.axis] += fb;
-    F[k] = L[0];
-    F[k + n] = L[1];
-    F[k + 2 * n] = L[2];
-}
-
-template <typename T>
-__device__ __forceinline__ T body_force_at(const ForceCoef<T>& c, long long t) {
-    const double fb_d = c.amp != 0.0 ? c.F0 * (1.0 + c.amp * sin(c.omega * (double)t)) : c.F0;
-    return (T)fb_d;
-}
-
-template <typename T, int DIM, int Q = kDefaultFlowQ<DIM>>
-__global__ void __launch_bounds__(256) k_force(Geo g, const T* __restrict__ b, T* __restrict__ F,
-                                               ForceCoef<T> c, const long long* __restrict__ tstep) {
-    const long long n = g.n;
-    const int nx = g.nx, ny = g.ny, nz = g.nz;
-    const T fb = body_force_at(c, *tstep);
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
-         k += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(k % nx);
-        const int y = (int)((k / nx) % ny);
-        const int z = (int)(k / ((long long)nx * ny));
-        force_node<T, DIM, Q>(b, F, n, nx, ny, nz, x, y, z, k, c, fb);
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Single-step flow update + IB on u, one z plane per CTA.  For each neighbour
-// y = x + c_j the equilibria of direction j (as f_j(x + c_j)) and of the
-// opposite direction (as f_jbar(x - c_jbar)) are formed from one load of y:
-//   drho* = 2 f~_0(x) - drho(x) + sum_j [ 0.5 f~_j(y) + 1.5 f~_jbar(y) ]
-//   m*    = sum_j c_j [ (tau - 1) f~_j(y) - tau f~_jbar(y) ] - 2 (tau - 1) rho u(x)
-//           - (tau/2) sum_j c_j [ F_j(y) + F_jbar(y) ] + F(x)
-// with f~_i = f_i^eq - w_i = w_i (drho + q_i + drho q_i),
-// q_i = 3 c_i.u + 4.5 (c_i.u)^2 - 1.5 u.u, and the GZS terms
-// F_j + F_jbar = (1 - 1/2tau) w_j (-6 u.F + 18 (c_j.u)(c_j.F)).  This uses
-// sum_i f_i^eq(x) = rho and sum_i c_i f_i^eq(x) = rho u, exact on the lattice.
-template <typename T, int DIM, int Q = kDefaultFlowQ<DIM>>
-__device__ __forceinline__ void flow_node(const T* __restrict__ drho, const T* __restrict__ u,
-                                          const T* __restrict__ F, T* __restrict__ drho_out, T* uout, long long n,
-                                          int nx, int ny, int nz, int x, int y, int z, long long k,
-                                          const FlowCoef<T>& c) {
-    const T* u1 = u + n;
-    const T* u2 = u + 2 * n;
-    const T* F1 = F + n;
-    const T* F2 = F + 2 * n;
-    const T tau = c.tau, tm1 = c.tau - T(1), half_tau = T(0.5) * c.tau;
-    const T dr0 = drho[k];
-    const T ux0 = u[k], uy0 = u[k + n], uz0 = u[k + 2 * n];
-    const T uu0 = ux0 * ux0 + uy0 * uy0 + uz0 * uz0;
-    const T q0 = T(-1.5) * uu0 * c.ig;
-    const T w0 = (T)flow_w<Q>(0);
-    // single-step density (Sec. III.E) or the macroscopic scheme's (Sec. V.G);
-    // c.mac is uniform across the launch
-    T rho_acc = c.mac ? w0 * (dr0 + q0 + dr0 * q0) : T(2) * w0 * (dr0 + q0 + dr0 * q0) - dr0;
-    T m[3] = {T(0), T(0), T(0)};
-    T corr[3] = {T(0), T(0), T(0)};
-#pragma unroll
-    for (int j = 1; j < Q; ++j) {
-        int cx, cy, cz;
-        flow_dir<Q>(j, cx, cy, cz);
-        const int q = (wrapi(z + cz, nz) * ny + wrapi(y + cy, ny)) * nx + wrapi(x + cx, nx);
-        const T dr = drho[q];
-        const T uq[3] = {u[q], u1[q], u2[q]};
-        const T Fq[3] = {F[q], F1[q], F2[q]};
-        const T a = (T)cx * uq[0] + (T)cy * uq[1] + (T)cz * uq[2];
-        const T uu = uq[0] * uq[0] + uq[1] * uq[1] + uq[2] * uq[2];
-        const T cF = (T)cx * Fq[0] + (T)cy * Fq[1] + (T)cz * Fq[2];
-        const T uF = uq[0] * Fq[0] + uq[1] * Fq[1] + uq[2] * Fq[2];
-        const T w = (T)flow_w<Q>(j);
-        const T sq = (T(4.5) * a * a - T(1.5) * uu) * c.ig;
-        const T qp = T(3) * a + sq, qm = T(-3) * a + sq;
-        const T fj = w * (dr + qp + dr * qp);
-        const T fjb = w * (dr + qm + dr * qm);
-        if (c.mac)
-            rho_acc += fjb;  // f^eq of direction -c_j at x + c_j
-        else
-            rho_acc += T(0.5) * fj + T(1.5) * fjb;
-        const T mom = tm1 * fj - tau * fjb;
-        const T fs = c.kforce * w * (T(-6) * uF + T(18) * a * cF) * c.ig2;
-        if (cx) {
-            m[0] += (T)cx * mom;
-            corr[0] += (T)cx * fs;
-        }
-        if (cy) {
-            m[1] += (T)cy * mom;
-            corr[1] += (T)cy * fs;
-        }
-        if (cz) {
-            m[2] += (T)cz * mom;
-            corr[2] += (T)cz * fs;
-        }
-    }
-    const T rho0 = T(1) + dr0;
-    const T rho_new = T(1) + rho_acc;
-    const T inv = T(1) / rho_new;
-    const T Fk[3] = {F[k], F[k + n], F[k + 2 * n]};
-    const T u0v[3] = {ux0, uy0, uz0};
-    drho_out[k] = rho_acc;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const T mm = m[a] - T(2) * tm1 * rho0 * u0v[a] - half_tau * corr[a] + Fk[a] * c.ig;
-        uout[k + a * n] = mm * inv;
-    }
-}
-
-template <typename T, int DIM, int Q = kDefaultFlowQ<DIM>>
-__global__ void __launch_bounds__(kPlaneThreads) k_flow_ib(Geo g, const T* __restrict__ drho,
-                                                           const T* __restrict__ u, const T* __restrict__ F,
-                                                           T* __restrict__ drho_out, T* uout, FlowCoef<T> c,
-                                                           IBView<T> ib, long long* tstep) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* sdelta = reinterpret_cast<T*>(smem_raw);
-    const int nx = g.nx, ny = g.ny, nz = g.nz;
-    const int z = blockIdx.x;
-    const long long n = g.n;
-    const long long P = (long long)nx * ny;
-    const long long base = (long long)z * P;
-    for (int p = threadIdx.x; p < P; p += blockDim.x) {
-        const int y = p / nx;
-        const int x = p - y * nx;
-        flow_node<T, DIM, Q>(drho, u, F, drho_out, uout, n, nx, ny, nz, x, y, z, base + p, c);
-    }
-    ib_plane<T>(ib, uout, uout + n, uout + 2 * n, base, ib.zinv ? 0 : z, sdelta);
-    if (blockIdx.x == 0 && threadIdx.x == 0) *tstep += 1;
-}
-
-// ---------------------------------------------------------------------------
 // Initial state: drho = 0, b = 0, u = splitmix64 noise (Steele, Lea, Flood)
 // of the counter seed ^ (3 k + component), top 53 bits to [-1, 1), times amp,
 // on nodes within radius R of the wall centre (between the walls for a channel).

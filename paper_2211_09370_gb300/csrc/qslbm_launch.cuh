@@ -6,6 +6,7 @@
 
 #include "qslbm_fused.cuh"
 #include "qslbm_internal.h"
+#include "qslbm_flow.cuh"
 #include "qslbm_kernels.cuh"
 #include "qslbm_resident.cuh"
 #include "qslbm_resident64.cuh"
@@ -78,6 +79,37 @@ struct Launch {
                                                        s.units.U0, s.axis);
     }
 
+    // The staged IB corrector on every plane of f.
+    static void launch_ib_staged(const State& s, T* f, const IBView<T>& v, cudaStream_t st) {
+        const int R = s.ib.max_ring, S = s.ib.max_shell;
+        const size_t sm = s.ib_staged_smem;
+        const dim3 ig((unsigned)s.nz), ib(kNodeThreads);
+        switch (s.ib_staged_u) {
+            case 1: launch_pdl(k_ib_staged<T, 1>, ig, ib, sm, st, geo(s), f, v, R, S); break;
+            case 2: launch_pdl(k_ib_staged<T, 2>, ig, ib, sm, st, geo(s), f, v, R, S); break;
+            case 4: launch_pdl(k_ib_staged<T, 4>, ig, ib, sm, st, geo(s), f, v, R, S); break;
+            default: launch_pdl(k_ib_staged<T, 5>, ig, ib, sm, st, geo(s), f, v, R, S); break;
+        }
+    }
+
+    // Planes per CTA of the marching force and flow kernels: two extra planes are
+    // read per chunk, and a chunk as long as leaves every SM some CTAs hides them.
+    static int flow_chunk(const State& s) {
+        const long long tiles = (long long)((s.nx + kFlowTX - 1) / kFlowTX) * ((s.ny + kFlowTY<T> - 1) / kFlowTY<T>);
+        const long long slots = 152LL * 4;
+        int best = 1;
+        long long cost = 1LL << 62;
+        for (int chunk = 1; chunk <= 32 && chunk <= s.nz; ++chunk) {
+            const long long waves = (tiles * ((s.nz + chunk - 1) / chunk) + slots - 1) / slots;
+            const long long c = waves * (chunk + 2);
+            if (c < cost) {
+                cost = c;
+                best = chunk;
+            }
+        }
+        return best;
+    }
+
     static void sweeps(State& s, int nsweeps, cudaStream_t st) {
         SweepCoef<T> c;
         sweep_weights(s, c.w0, c.w1, c.kappa);
@@ -131,15 +163,7 @@ struct Launch {
                     k_sweep_nodes<T, 2><<<grid, kNodeThreads, 0, st>>>(geo(s), bin, bout, u, c);
                 }
                 if (s.ib.nm > 0 && s.ib_staged_smem > 0) {
-                    const int R = s.ib.max_ring, S = s.ib.max_shell;
-                    const size_t sm = s.ib_staged_smem;
-                    const dim3 ig((unsigned)s.nz), ib(kNodeThreads);
-                    switch (s.ib_staged_u) {
-                        case 1: launch_pdl(k_ib_staged<T, 1>, ig, ib, sm, st, geo(s), bout, v, R, S); break;
-                        case 2: launch_pdl(k_ib_staged<T, 2>, ig, ib, sm, st, geo(s), bout, v, R, S); break;
-                        case 4: launch_pdl(k_ib_staged<T, 4>, ig, ib, sm, st, geo(s), bout, v, R, S); break;
-                        default: launch_pdl(k_ib_staged<T, 5>, ig, ib, sm, st, geo(s), bout, v, R, S); break;
-                    }
+                    launch_ib_staged(s, bout, v, st);
                 } else if (s.ib.nm > 0) {
                     k_ib_markers<T><<<(s.ib.nm + kNodeThreads - 1) / kNodeThreads, kNodeThreads, 0, st>>>(geo(s), bout, v);
                     k_ib_shell<T><<<(s.ib.ns + kNodeThreads - 1) / kNodeThreads, kNodeThreads, 0, st>>>(geo(s), bout, v);
@@ -723,16 +747,27 @@ struct Launch {
         T* dro = (T*)s.drho[1 - s.fcur];
         T* uo = (T*)s.u[1 - s.fcur];
         T* F = (T*)s.F;
-        if (s.dim == 3 && s.units.flow_q == 27) {
-            k_force<T, 3, 27><<<grid_for(s.n, 256), 256, 0, st>>>(geo(s), b, F, fc, s.tdev);
-            k_flow_ib<T, 3, 27><<<s.nz, kPlaneThreads, ib_smem(s), st>>>(geo(s), dr, u, F, dro, uo, c, v, s.tdev);
-        } else if (s.dim == 3) {
-            k_force<T, 3><<<grid_for(s.n, 256), 256, 0, st>>>(geo(s), b, F, fc, s.tdev);
-            k_flow_ib<T, 3><<<s.nz, kPlaneThreads, ib_smem(s), st>>>(geo(s), dr, u, F, dro, uo, c, v, s.tdev);
+        if (s.dim == 2) {
+            const int blocks = (s.nx * s.ny + kFlowNodeThreads - 1) / kFlowNodeThreads;
+            k_force_nodes<T, 9><<<blocks, kFlowNodeThreads, 0, st>>>(geo(s), b, F, fc, s.tdev);
+            k_flow_nodes<T, 9><<<blocks, kFlowNodeThreads, 0, st>>>(geo(s), dr, u, F, dro, uo, c, s.tdev);
         } else {
-            k_force<T, 2><<<grid_for(s.n, 256), 256, 0, st>>>(geo(s), b, F, fc, s.tdev);
-            k_flow_ib<T, 2><<<s.nz, kPlaneThreads, ib_smem(s), st>>>(geo(s), dr, u, F, dro, uo, c, v, s.tdev);
+            const int chunk = flow_chunk(s);
+            const dim3 grid((unsigned)((s.nx + kFlowTX - 1) / kFlowTX),
+                            (unsigned)((s.ny + kFlowTY<T> - 1) / kFlowTY<T>), (unsigned)((s.nz + chunk - 1) / chunk));
+            constexpr int threads = kFlowThreads<T>;
+            if (s.units.flow_q == 27) {
+                k_force_march<T, 27><<<grid, threads, 0, st>>>(geo(s), b, F, fc, s.tdev, chunk);
+                k_flow_march<T, 27><<<grid, threads, 0, st>>>(geo(s), dr, u, F, dro, uo, c, s.tdev, chunk);
+            } else {
+                k_force_march<T, 19><<<grid, threads, 0, st>>>(geo(s), b, F, fc, s.tdev, chunk);
+                k_flow_march<T, 19><<<grid, threads, 0, st>>>(geo(s), dr, u, F, dro, uo, c, s.tdev, chunk);
+            }
         }
+        if (s.ib.nm > 0 && s.ib_staged_smem > 0)
+            launch_ib_staged(s, uo, v, st);
+        else if (s.ib.nm > 0)
+            k_ib_planes<T><<<s.nz, kNodeThreads, ib_smem(s), st>>>(geo(s), uo, v);
         s.fcur ^= 1;
     }
 
