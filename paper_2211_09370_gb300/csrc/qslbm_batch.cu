@@ -510,8 +510,7 @@ int build_groups(qslbm_batch& B) {
     BCHK(cudaMemsetAsync(B.xbuf, 0, sizeof(uint4) * xoff, B.stream));
     BCHK(cudaMemsetAsync(B.gerr, 0, sizeof(int), B.stream));
     for (bool xy : {false, true})
-        BCHK(cudaFuncSetAttribute((const void*)group_kernel(B.gstride, xy),
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        BCHK(qslbm::allow_smem((const void*)group_kernel(B.gstride, xy), smem));
     return QSLBM_OK;
 }
 
@@ -577,14 +576,10 @@ int build_tables(qslbm_batch& B, int threads) {
         BCHK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
         if (smem <= (size_t)optin) {
             // the launch picks U per active set (ib_staged_unroll)
-            BCHK(cudaFuncSetAttribute(qslbm::k_batch_ib_staged<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
-            BCHK(cudaFuncSetAttribute(qslbm::k_batch_ib_staged<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
-            BCHK(cudaFuncSetAttribute(qslbm::k_batch_ib_staged<T, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
-            BCHK(cudaFuncSetAttribute(qslbm::k_batch_ib_staged<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
+            BCHK(qslbm::allow_smem((const void*)qslbm::k_batch_ib_staged<T, 1>, smem));
+            BCHK(qslbm::allow_smem((const void*)qslbm::k_batch_ib_staged<T, 2>, smem));
+            BCHK(qslbm::allow_smem((const void*)qslbm::k_batch_ib_staged<T, 5>, smem));
+            BCHK(qslbm::allow_smem((const void*)qslbm::k_batch_ib_staged<T, 4>, smem));
             B.ib_staged_smem = smem;
         }
     }
@@ -780,7 +775,7 @@ int group_capacity(qslbm_batch& B) {
     cudaFuncAttributes fa;
     BCHK(cudaFuncGetAttributes(&fa, fn));
     optin -= (int)fa.sharedSizeBytes;
-    BCHK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
+    BCHK(qslbm::allow_smem(fn, optin));
     BCHK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, qslbm::kGroupThreads, optin));
     B.gcap = occ * sms;
     B.goptin = optin;

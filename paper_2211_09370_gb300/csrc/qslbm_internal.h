@@ -4,12 +4,26 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <mutex>
 #include <string>
 #include <vector>
 
 #include "qslbm.h"
 
 namespace qslbm {
+
+// Allows kernel fn to launch with `bytes` of dynamic shared memory.  The limit is the
+// process's, shared by every handle and batch that launches fn, and it is enforced
+// downwards too: it only ever rises here, or a small handle made after a large one
+// would have the large one's launches refused.
+inline cudaError_t allow_smem(const void* fn, size_t bytes) {
+    static std::mutex m;
+    const std::lock_guard<std::mutex> lock(m);
+    cudaFuncAttributes fa;
+    const cudaError_t e = cudaFuncGetAttributes(&fa, fn);
+    if (e != cudaSuccess || (size_t)fa.maxDynamicSharedSizeBytes >= bytes) return e;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
 
 // Diagnostics slots and the reduction block size (see k_observe).
 constexpr int kObs = 11;

@@ -264,7 +264,7 @@ struct Launch {
             const int pairs = (s.fu_TY + 4) * s.nx / 2;
             s.fu_threads = std::min(kFusedMaxThreads, (pairs + 31) / 32 * 32);
             auto kern = fused_kernel(s);
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.fu_smem);
+            cudaError_t e = allow_smem((const void*)kern, s.fu_smem);
             if (e != cudaSuccess) {
                 cudaGetLastError();
                 s.fused = false;
@@ -390,7 +390,7 @@ struct Launch {
         const size_t smem = slab_direct_smem_bytes(s.nx, s.ny, G, R, S, more);
         if (smem + 1024 > (size_t)optin) return cudaSuccess;
         const auto kern = slab_kernel(K);
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem((const void*)kern, smem);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return cudaSuccess;
@@ -489,8 +489,8 @@ struct Launch {
         ok = false;
         auto kern = k_sweeps_resident<T, DIM, UHALO, RT, NPT, false>;
         auto kern2 = k_sweeps_resident<T, DIM, UHALO, RT, NPT, true>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem((const void*)kern, smem);
+        if (e == cudaSuccess) e = allow_smem((const void*)kern2, smem);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return cudaSuccess;  // too much shared memory: not resident
@@ -557,11 +557,11 @@ struct Launch {
             if (smem <= (size_t)max_optin) {
                 s.ib_staged_u = ib_staged_unroll(s.ib.max_shell, s.nz, sms);
                 const int U = s.ib_staged_u;
-                e = cudaFuncSetAttribute(U == 1   ? k_ib_staged<T, 1>
-                                         : U == 2 ? k_ib_staged<T, 2>
-                                         : U == 4 ? k_ib_staged<T, 4>
-                                                  : k_ib_staged<T, 5>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                const auto kern = U == 1   ? k_ib_staged<T, 1>
+                                  : U == 2 ? k_ib_staged<T, 2>
+                                  : U == 4 ? k_ib_staged<T, 4>
+                                           : k_ib_staged<T, 5>;
+                e = allow_smem((const void*)kern, smem);
                 if (e != cudaSuccess) return e;
                 s.ib_staged_smem = smem;
             }
@@ -575,8 +575,7 @@ struct Launch {
         ok = false;
         if ((long long)s.nx * s.ny > (long long)kRes64Threads * kRes64MaxNpt) return cudaSuccess;
         const auto kern = resident64_kernel(s);
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess) {
+        if (allow_smem((const void*)kern, smem) != cudaSuccess) {
             cudaGetLastError();
             return cudaSuccess;
         }
@@ -623,7 +622,7 @@ struct Launch {
             cudaError_t e = cudaSuccess;
             if (C > 8) e = cudaFuncSetAttribute(k_sweeps_cluster64<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
             if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_sweeps_cluster64<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                e = allow_smem((const void*)k_sweeps_cluster64<T>, smem);
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3((unsigned)C);
             cfg.blockDim = dim3(kC2Threads);
