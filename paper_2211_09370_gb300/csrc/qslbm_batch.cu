@@ -2,10 +2,12 @@
 // advance together, every phase of a flow step being one fused launch over all
 // instances' work.  The time loop is captured into a CUDA graph (one graph per
 // step, replayed); ping-pong parities live in device memory so the same graph
-// serves every step.  Instances are ordered by N_mag (descending): sweep s only
-// touches the prefix of instances with N_mag > s.  The node-parallel sweep
-// kernel is persistent (grid-stride over the work list) with its block size
-// and grid chosen by a timing autotuner when the batch is built.
+// serves every step.  An instance's sweeps take one of three routes: the resident
+// groups (qslbm_groups.cuh), a chain of its own kernels on a side stream, or the
+// joint march, whose instances are ordered by N_mag (descending): sweep s only
+// touches the prefix of instances with N_mag > s, with a persistent kernel
+// (grid-stride over the work list) whose block size and grid a timing autotuner
+// chooses when the batch is first built with such an instance.
 //
 // The per-node arithmetic is the single-instance code (march_tile, the IB sums
 // of ib_plane, force_gather, flow_gather), so a batched instance follows the same
@@ -129,6 +131,31 @@ __global__ void __launch_bounds__(kNodeThreads, (kIbStagedMinBlocks<T, U>)) k_ba
                                      max_shell, smem_raw);
 }
 
+// Sweep s of one member alone, on node pairs, and its IB pass: the two kernels of its
+// chain (launch_chain).  D: the member, of which the parities are
+// read where they advance (live).
+template <bool XY>
+__global__ void __launch_bounds__(kPairThreads, 3) k_chain_sweep(InstDesc<float> D, const InstDesc<float>* live,
+                                                                 int s, int chunk) {
+    __shared__ __align__(16) PairTile tile;
+    pdl_trigger();
+    pdl_wait();
+    const int par = (live->bpar + s) & 1;
+    const float* u = live->fpar ? D.u[1] : D.u[0];
+    pair_tile<XY>(D.g, par ? D.b[1] : D.b[0], par ? D.b[0] : D.b[1], u, D.sc, blockIdx.x, blockIdx.y, blockIdx.z, chunk, tile);
+}
+template <int U>
+__global__ void __launch_bounds__(kNodeThreads, (kIbStagedMinBlocks<float, U>))
+    k_chain_ib(Geo g, float* b0, float* b1, IBView<float> ib, const InstDesc<float>* live, int s, int max_ring,
+               int max_shell) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_trigger();
+    const int z = blockIdx.x;
+    ib_staged_plane<float, kNodeThreads, U, (U == 2 || U == 4)>(ib, ((live->bpar + s) & 1) ? b0 : b1, (int)g.n,
+                                                                z * g.nx * g.ny, ib.zinv ? 0 : z, max_ring, max_shell,
+                                                                smem_raw);
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kNodeThreads) k_batch_ib(const InstDesc<T>* __restrict__ d,
                                                            const int* __restrict__ pfirst, int kact, int s) {
@@ -201,7 +228,7 @@ __global__ void k_batch_advance(InstDesc<T>* d, int k) {
 using qslbm::State;
 
 struct qslbm_batch {
-    std::vector<qslbm_handle*> members;  // marching members by N_mag (descending), then the resident groups' members
+    std::vector<qslbm_handle*> members;  // jointly marching members by N_mag (descending), chains', resident groups'
     std::vector<int> order;              // order[k] = caller's index of member k
     std::vector<int> rank;               // rank[caller index] = k
     cudaStream_t stream = nullptr;
@@ -234,7 +261,13 @@ struct qslbm_batch {
     long long steps = 0;
     long long device_bytes = 0;
     std::vector<double> tune_us;         // timing of each candidate
-    // resident groups (FP32): members [kmarch, K) run all their sweeps in one
+    // chains (FP32): members [kmarch, kgroup) sweep each in a chain of its own
+    // kernels, concurrently on side streams (launch_chains)
+    int kgroup = 0;
+    std::vector<cudaStream_t> side;
+    std::vector<cudaEvent_t> joined;
+    cudaEvent_t forked = nullptr;
+    // resident groups (FP32): members [kgroup, K) run all their sweeps in one
     // cooperative launch of k_batch_resident, a group of whole planes per CTA
     int kmarch = 0;
     std::vector<int> gplanes;            // per member: planes per group (0: marching)
@@ -423,10 +456,81 @@ void launch_groups(qslbm_batch& B, cudaStream_t st) {
     }
 }
 
+// A marching member of an FP32 batch in a chain of its own kernels: the pair sweep on
+// a grid of one wave and its IB pass, which run concurrently with the other chains.
+// Both kernels are bound by latency (the sweep issues in 39 % of the cycles), so
+// that members' kernels fill each other's stalls, tails and launch gaps; in the joint
+// march every sweep waits for the whole batch twice, and tiles of one row a thread
+// cost more.  Us a sweep, joint / chains: eight pipes of 32x32x183 to 85x85x505 186 /
+// 146; one 96x96x512 67.7 / 51.6, three 88x88x300 108 / 75, four 72x72x200 79.5 /
+// 54.9, six 48x48x180 49.0 / 36.1, eight 40x40x130 39.0 / 30.1, nine 32x32x100 19.8 /
+// 12.3; nothing smaller was measured.  At most kChains of them, the largest, with a
+// stream each (a graph of a step holds 2 N_mag nodes per chain).
+constexpr int kChains = 16;
+constexpr long long kChainNodes = 100000;
+
+bool chain_member(const State& s) {
+    return s.esz == 4 && s.dim == 3 && s.n >= kChainNodes && (s.ib.nm == 0 || s.ib_staged_smem > 0);
+}
+
+void launch_chain(qslbm_batch& B, int k, cudaStream_t st) {
+    const State& s = qslbm::handle_state_mut(B.members[k]);
+    const auto* live = (const qslbm::InstDesc<float>*)B.desc + k;
+    const qslbm::InstDesc<float> D = make_desc<float>(s);
+    const dim3 grid((unsigned)((s.nx + 2 * qslbm::kPairTXP - 1) / (2 * qslbm::kPairTXP)),
+                    (unsigned)((s.ny + qslbm::kPairTY - 1) / qslbm::kPairTY),
+                    (unsigned)((s.nz + s.march_chunk - 1) / s.march_chunk));
+    const int R = s.ib.max_ring, S = s.ib.max_shell;
+    const dim3 ig((unsigned)s.nz), ib(qslbm::kNodeThreads);
+    for (int i = 0; i < s.units.n_mag; ++i) {
+        // (the first waits for the kernels before the step's sweeps in full)
+        launch_pdl(i > 0, s.bext_xy ? qslbm::k_chain_sweep<true> : qslbm::k_chain_sweep<false>, grid,
+                   dim3(qslbm::kPairThreads), 0, st, D, live, i, s.march_chunk);
+        if (s.ib.nm == 0) continue;
+        const auto kern = s.ib_staged_u == 1   ? qslbm::k_chain_ib<1>
+                          : s.ib_staged_u == 2 ? qslbm::k_chain_ib<2>
+                          : s.ib_staged_u == 4 ? qslbm::k_chain_ib<4>
+                                               : qslbm::k_chain_ib<5>;
+        launch_pdl(true, kern, ig, ib, s.ib_staged_smem, st, D.g, D.b[0], D.b[1], D.ibm, live, i, R, S);
+    }
+}
+
+// Streams and shared-memory limits for the chains of the members [kmarch, kgroup).
+int prepare_chains(qslbm_batch& B) {
+    const size_t n = (size_t)(B.kgroup - B.kmarch);
+    if (n > 0 && !B.forked) BCHK(cudaEventCreateWithFlags(&B.forked, cudaEventDisableTiming));
+    while (B.side.size() < n) {
+        cudaStream_t st = nullptr;
+        cudaEvent_t e = nullptr;
+        BCHK(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+        B.side.push_back(st);
+        BCHK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        B.joined.push_back(e);
+    }
+    for (int k = B.kmarch; k < B.kgroup; ++k) {
+        const State& s = qslbm::handle_state_mut(B.members[k]);
+        if (s.ib.nm == 0) continue;
+        BCHK(qslbm::allow_smem((const void*)qslbm::k_chain_ib<1>, s.ib_staged_smem));
+        BCHK(qslbm::allow_smem((const void*)qslbm::k_chain_ib<2>, s.ib_staged_smem));
+        BCHK(qslbm::allow_smem((const void*)qslbm::k_chain_ib<4>, s.ib_staged_smem));
+        BCHK(qslbm::allow_smem((const void*)qslbm::k_chain_ib<5>, s.ib_staged_smem));
+    }
+    return QSLBM_OK;
+}
+
 template <typename T>
 void launch_step(qslbm_batch& B, cudaStream_t st) {
     launch_groups<T>(B, st);
+    // the chains beside the joint sweeps of the other marching members
+    const int nc = B.kgroup - B.kmarch;
+    if (nc > 0) cudaEventRecord(B.forked, st);
+    for (int j = 0; j < nc; ++j) {
+        cudaStreamWaitEvent(B.side[j], B.forked, 0);
+        launch_chain(B, B.kmarch + j, B.side[j]);
+        cudaEventRecord(B.joined[j], B.side[j]);
+    }
     for (int s = 0; s < B.max_nmag; ++s) launch_sweep<T>(B, s, B.threads, B.grid, st);
+    for (int j = 0; j < nc; ++j) cudaStreamWaitEvent(st, B.joined[j], 0);  // (an error ends the graph capture)
     const int K = (int)B.members.size();
     auto* d = (qslbm::InstDesc<T>*)B.desc;
     qslbm::k_batch_force<T><<<B.h_pfirst[K], qslbm::kNodeThreads, 0, st>>>(d, B.pfirst, K);
@@ -461,7 +565,7 @@ int build_groups(qslbm_batch& B) {
     B.h_groups.clear();
     long long xoff = 0;
     size_t smem = 0;
-    for (int k = B.kmarch; k < K; ++k) {
+    for (int k = B.kgroup; k < K; ++k) {
         const State& s = qslbm::handle_state_mut(B.members[k]);
         const int P = s.nx * s.ny;
         const int ng = group_count(s, B.gplanes[k]);
@@ -690,11 +794,15 @@ int capture_steps(qslbm_batch& B, int steps, cudaGraphExec_t* out) {
 }
 
 // Launches of one flow step: the group kernel, each marching sweep with its
-// IB pass (or two), force, flow, parity advance.
+// IB pass (or two), the chains' likewise, force, flow, parity advance.
 int step_launches(const qslbm_batch& B) {
     int n = 3 + (B.ngroups > 0 ? 1 : 0);
     for (int s = 0; s < B.max_nmag; ++s)
         if (B.active[s] > 0) n += 1 + (B.h_mfirst[B.active[s]] > 0 ? (B.ib_staged_smem ? 1 : 2) : 0);
+    for (int k = B.kmarch; k < B.kgroup; ++k) {
+        const State& s = qslbm::handle_state_mut(B.members[k]);
+        n += s.units.n_mag * (s.ib.nm > 0 ? 2 : 1);
+    }
     return n;
 }
 
@@ -756,6 +864,9 @@ void destroy_batch(qslbm_batch* B) {
     if (B->pfirst) cudaFree(B->pfirst);
     if (B->mfirst) cudaFree(B->mfirst);
     if (B->sfirst) cudaFree(B->sfirst);
+    for (cudaStream_t st : B->side) cudaStreamDestroy(st);
+    for (cudaEvent_t e : B->joined) cudaEventDestroy(e);
+    if (B->forked) cudaEventDestroy(B->forked);
     if (B->owns_members)
         for (qslbm_handle* h : B->members) qslbm_destroy(h);
     if (B->own_stream && B->stream) cudaStreamDestroy(B->stream);
@@ -795,7 +906,7 @@ int set_members(qslbm_batch* B, const std::vector<qslbm_handle*>& hs, const std:
     B->order.assign(count, 0);
     B->rank.assign(count, 0);
     B->gplanes.clear();
-    B->kmarch = 0;
+    B->kmarch = B->kgroup = 0;
     B->ngroups = 0;
     if (count == 0) {
         if (B->graph) {
@@ -876,10 +987,24 @@ int set_members(qslbm_batch* B, const std::vector<qslbm_handle*>& hs, const std:
         for (int i : adm) spread[i] = planes_at(i, lo);
         for (int i : adm) gp[i] = spread[i];
     }
+    // chains: the marching members of some size (FP32), the largest first
+    std::vector<char> chain(count, 0);
+    if (B->precision == QSLBM_FP32) {
+        std::vector<int> big;
+        for (int i = 0; i < count; ++i)
+            if (gp[i] == 0 && chain_member(qslbm::handle_state_mut(hs[i]))) big.push_back(i);
+        std::stable_sort(big.begin(), big.end(), [&](int a, int b) {
+            return qslbm::handle_state_mut(hs[a]).n > qslbm::handle_state_mut(hs[b]).n;
+        });
+        if (big.size() > kChains) big.resize(kChains);
+        for (int i : big) chain[i] = 1;
+    }
     std::vector<int> idx(count);
     std::iota(idx.begin(), idx.end(), 0);
+    // jointly marching members first, then the chains', then the groups'
+    auto kind = [&](int i) { return gp[i] > 0 ? 2 : (chain[i] ? 1 : 0); };
     std::stable_sort(idx.begin(), idx.end(), [&](int a, int b) {
-        if ((gp[a] > 0) != (gp[b] > 0)) return gp[b] > 0;  // marching members first
+        if (kind(a) != kind(b)) return kind(a) < kind(b);
         return qslbm::handle_state_mut(hs[a]).units.n_mag > qslbm::handle_state_mut(hs[b]).units.n_mag;
     });
     B->order = idx;
@@ -887,7 +1012,8 @@ int set_members(qslbm_batch* B, const std::vector<qslbm_handle*>& hs, const std:
         B->members.push_back(hs[idx[k]]);
         B->rank[idx[k]] = k;
         B->gplanes.push_back(gp[idx[k]]);
-        if (gp[idx[k]] == 0) B->kmarch = k + 1;
+        if (kind(idx[k]) == 0) B->kmarch = k + 1;
+        if (kind(idx[k]) <= 1) B->kgroup = k + 1;
     }
     B->max_nmag = 0;
     for (qslbm_handle* h : B->members) B->max_nmag = std::max(B->max_nmag, qslbm::handle_state_mut(h).units.n_mag);
@@ -898,7 +1024,8 @@ int set_members(qslbm_batch* B, const std::vector<qslbm_handle*>& hs, const std:
         while (a < B->kmarch && qslbm::handle_state_mut(B->members[a]).units.n_mag > s) ++a;
         B->active[s] = a;
     }
-    int rc;
+    int rc = prepare_chains(*B);
+    if (rc) return rc;
     if (!B->tuned && B->kmarch > 0) {  // (no marching member: nothing to time yet)
         rc = B->precision == QSLBM_FP64 ? autotune<double>(*B) : autotune<float>(*B);
         B->tuned = true;
@@ -1015,7 +1142,7 @@ int qslbm_batch_info(const qslbm_batch* B, qslbm_batch_info_t* info) {
     info->node_sweeps_per_step = sweeps;
     info->device_bytes = bytes;
     info->launches_per_step = B->members.empty() ? 0 : step_launches(*B);
-    info->resident_instances = (int32_t)B->members.size() - B->kmarch;
+    info->resident_instances = (int32_t)B->members.size() - B->kgroup;
     info->resident_groups = B->ngroups;
     info->graph_steps = B->chunk_steps;
     info->march_chunk = B->chunk;
