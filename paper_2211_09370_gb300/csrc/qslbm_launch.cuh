@@ -413,7 +413,7 @@ struct Launch {
     }
 
     static auto resident64_kernel(const State& s) {
-        return s.nx * s.ny <= 4 * kRes64Threads ? k_sweeps_resident64<T, 4> : k_sweeps_resident64<T, kRes64MaxNpt>;
+        return s.nx * s.ny <= 8 * kRes64Threads ? k_sweeps_resident64<T, 8> : k_sweeps_resident64<T, kRes64MaxNpt>;
     }
 
     // FP64: one plane per CTA in 3-D, one thread-block cluster in 2-D.
@@ -435,7 +435,7 @@ struct Launch {
             attr[0].id = cudaLaunchAttributeCooperative;
             attr[0].val.cooperative = 1;
             e = cudaLaunchKernelEx(&cfg, resident64_kernel(s), geo(s), bin, bout, u, c, v, (T*)s.xbuf,
-                                   (ResidentSync*)s.rsync, nsweeps, s.ib.max_ring, s.ib.max_shell, s.ib.max_nnz);
+                                   (ResidentSync*)s.rsync, nsweeps, s.ib.max_ring, s.ib.max_shell);
         } else {
             cfg.gridDim = dim3((unsigned)s.c2_ctas);
             cfg.blockDim = dim3(kC2Threads);
@@ -693,10 +693,11 @@ struct Launch {
             } else {
                 int sms = 0;
                 if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-                if (base + reserve > (size_t)optin) return cudaSuccess;
-                if ((e = try_resident64(s, base, sms, ok)) != cudaSuccess) return e;
+                const size_t smem = resident64_smem_bytes((int)P, s.ib.max_ring, s.ib.max_shell, s.ib.max_nnz);
+                if (smem + reserve > (size_t)optin) return cudaSuccess;
+                if ((e = try_resident64(s, smem, sms, ok)) != cudaSuccess) return e;
                 s.resident = ok;
-                s.resident_smem = base;
+                s.resident_smem = smem;
                 return cudaSuccess;
             }
         }

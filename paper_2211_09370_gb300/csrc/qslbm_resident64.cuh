@@ -23,19 +23,29 @@ namespace qslbm {
 // counters; the z terms from the neighbours' (b, e2, e3) of the previous
 // sweep, a double-buffered exchange array in global memory (10 loads a node
 // instead of forming e twice more, 8 operations); the plane-local IB; the new
-// e of every node and its publication.  Operations left at 2 per clock: 42 x
-// 4096 nodes is 42 us a sweep for the 64x64x128 pipe.
-constexpr int kRes64Threads = 1024;
+// e of every node and its publication.  Operations at 2 per clock: 42 x 4096 nodes
+// is 42 us a sweep for the 64x64x128 pipe, which takes 55.3 us (the marching sweep
+// and its IB 65.6; 65x65x120 57.6 against 96.3, 48x48x128 32.7 against 55.8).  512
+// threads keep the FP64 pipe as busy as 1024 do and have the registers for the new
+// values of their nodes (1024, which spilled them: 57.7).
+constexpr int kRes64Threads = 512;
 // nodes per thread, at most: planes whose b and e fit shared memory have at most
-// 4842; planes of up to 4096 take four (the fifth costs spills)
-constexpr int kRes64MaxNpt = 5;
+// 4842; planes of up to 4096 take eight (ten cost a few spills)
+constexpr int kRes64MaxNpt = 10;
 constexpr int kRes64Fields = 5;  // exchanged per node: b, e2, e3
+
+// Shared memory of a plane of P nodes with a ring of R markers, S shell nodes and E
+// list entries.  The weights are kept once, with 16-bit indices (48 B a node leave 35
+// KB of tables at 64x64, where separate weights and 32-bit indices took 44).
+inline size_t resident64_smem_bytes(int P, int R, int S, int E) {
+    return ((size_t)6 * P + 13 * R) * sizeof(double) + ((size_t)9 * R + 2 * S + 1 + E) * sizeof(unsigned short);
+}
 
 template <typename T, int kRes64Npt>
 __global__ void __launch_bounds__(kRes64Threads, 1)
     k_sweeps_resident64(Geo g, const T* __restrict__ b_in, T* __restrict__ b_out, const T* __restrict__ u,
                         SweepCoef<T> c, IBView<T> ib, T* xbuf, ResidentSync* sync, int nsweeps, int max_ring,
-                        int max_shell, int max_nnz) {
+                        int max_shell) {
     static_assert(sizeof(T) == 8, "the FP64 path");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ unsigned int s_epoch;
@@ -51,11 +61,12 @@ __global__ void __launch_bounds__(kRes64Threads, 1)
     double* sdelta = se + 3 * P;                       // [3 R]
     double* tw = sdelta + 3 * max_ring;                // [9 R]
     double* tsc = tw + 9 * max_ring;                   // [R]
-    double* tcw = tsc + max_ring;                      // [E]
-    int* tq = reinterpret_cast<int*>(tcw + max_nnz);   // [9 R]
-    int* tshell = tq + 9 * max_ring;                   // [S]
-    int* toff = tshell + max_shell;                    // [S + 1]
-    int* tcm = toff + max_shell + 1;                   // [E]
+    // 16 bits reach every index: a plane has at most 4842 nodes, and fewer list
+    // entries than that fit
+    unsigned short* tq = reinterpret_cast<unsigned short*>(tsc + max_ring);  // [9 R] support (in-plane index)
+    unsigned short* tshell = tq + 9 * max_ring;                              // [S] shell nodes
+    unsigned short* toff = tshell + max_shell;                               // [S + 1] list offsets
+    unsigned short* tl = toff + max_shell + 1;                               // [E] the markers' entries (of tw, tq)
     if (tid == 0) {
         s_epoch = *(volatile unsigned int*)&sync->epoch;
         s_abort = 0;
@@ -65,18 +76,26 @@ __global__ void __launch_bounds__(kRes64Threads, 1)
     const int s0 = ib.shell_off[tz], S = ib.shell_off[tz + 1] - s0;
     {
         const int e0 = S > 0 ? ib.csr_off[s0] : 0;
-        const int E = S > 0 ? ib.csr_off[s0 + S] - e0 : 0;
         for (int i = tid; i < 9 * R; i += kRes64Threads) {
-            tq[i] = ib.mk_q[9 * m0 + i];
+            tq[i] = (unsigned short)ib.mk_q[9 * m0 + i];
             tw[i] = ib.mk_w[9 * m0 + i];
         }
         for (int i = tid; i < R; i += kRes64Threads) tsc[i] = ib.mk_s[m0 + i];
-        for (int i = tid; i < S; i += kRes64Threads) tshell[i] = ib.shell_xy[s0 + i];
-        if (S > 0)
-            for (int i = tid; i <= S; i += kRes64Threads) toff[i] = ib.csr_off[s0 + i] - e0;
-        for (int i = tid; i < E; i += kRes64Threads) {
-            tcm[i] = ib.csr_m[e0 + i];
-            tcw[i] = ib.csr_w[e0 + i];
+        __syncthreads();
+        // a list entry is a marker's weight at the node: named by its place in tw
+        for (int i = tid; i < S; i += kRes64Threads) {
+            const int q = ib.shell_xy[s0 + i], o = ib.csr_off[s0 + i], o1 = ib.csr_off[s0 + i + 1];
+            tshell[i] = (unsigned short)q;
+            toff[i] = (unsigned short)(o - e0);
+            if (i == S - 1) toff[S] = (unsigned short)(o1 - e0);
+            for (int e = o; e < o1; ++e) {
+                const int m = ib.csr_m[e];
+                const double w = ib.csr_w[e];
+                int at = 9 * m;
+                for (int k = 9 * m; k < 9 * m + 9; ++k)
+                    if (tq[k] == q && tw[k] == w) at = k;
+                tl[e - e0] = (unsigned short)at;
+            }
         }
     }
     double be[3];
@@ -175,7 +194,10 @@ __global__ void __launch_bounds__(kRes64Threads, 1)
             for (int t = tid; t < 3 * S; t += kRes64Threads) {
                 const int i = t / 3, a = t - 3 * i;
                 double v = 0.0;
-                for (int e = toff[i]; e < toff[i + 1]; ++e) v = __fma_rn(tcw[e], sdelta[3 * tcm[e] + a], v);
+                for (int e = toff[i]; e < toff[i + 1]; ++e) {
+                    const int l = tl[e];
+                    v = __fma_rn(tw[l], sdelta[3 * (l / 9) + a], v);
+                }
                 sb[a * P + tshell[i]] += v;
             }
             __syncthreads();

@@ -69,3 +69,10 @@ BOXES = {
 @pytest.mark.parametrize("case", sorted(BOXES))
 def test_plane_kernel_matches_oracle(case):
     check(W.small_pipe(precision="fp64", n_mag=25, **BOXES[case]), 3)
+
+
+@pytest.mark.parametrize("case", ["4096_nodes", "above_4096_nodes"])
+def test_planes_at_the_limit_of_shared_memory(case):
+    # the IB tables in 16 bits, eight and nine or ten nodes per thread
+    n = dict(zip(["4096_nodes", "above_4096_nodes"], [(64, 64), (65, 65)]))[case]
+    check(W.small_pipe(nx=n[0], ny=n[1], nz=3, diameter=n[0] - 8.0, n_mag=9, precision="fp64", Ha=20.0, Rm=2e-3), 2)
