@@ -22,7 +22,8 @@
 // The sums run over the planes z - 1, z, z + 1 in turn (flow_plane), so that a CTA
 // can march through z with three targets' sums in registers; the gathering form
 // (flow_gather: 2-D, batched planes) adds in the same order.  Every rounding is
-// spelled out: the two forms agree to the bit.
+// spelled out: the two forms agree to the bit.  The node's own part of m*, its largest
+// term, is added last, so that the others' sum is not rounded at its size.
 #pragma once
 
 #include "qslbm_kernels.cuh"
@@ -118,24 +119,25 @@ __device__ __forceinline__ void flow_add(T s[4], int cx, int cy, int cz, const F
     if (cy) s[2] = fma_rn(cy > 0 ? w : -w, g, s[2]);
     if (cz) s[3] = fma_rn(cz > 0 ? w : -w, g, s[3]);
 }
-// The node itself: its own values v and (drho, u, F).
+// The node itself: its own values v and (drho, u, F); own: its part of m*.
 template <typename T, int Q>
-__device__ __forceinline__ void flow_own(T s[4], const FlowVals<T>& v, T dr, const T F[3], const FlowConst<T>& c) {
+__device__ __forceinline__ void flow_own(T s[4], T own[3], const FlowVals<T>& v, T dr, const T F[3],
+                                         const FlowConst<T>& c) {
     const T w0 = (T)flow_weight<Q>(0);
     s[0] = fma_rn(c.kappa * w0, v.K, s[0]);
     if (!c.mac) s[0] = add_rn(s[0], -dr);
     const T k = mul_rn(c.two_tm1, add_rn(T(1), dr));
 #pragma unroll
-    for (int a = 0; a < 3; ++a) s[1 + a] = fma_rn(c.ig, F[a], fma_rn(-k, v.u[a], s[1 + a]));
+    for (int a = 0; a < 3; ++a) own[a] = fma_rn(c.ig, F[a], -mul_rn(k, v.u[a]));
 }
 // Neighbour i of a plane (its place in-plane: flow_px, flow_py), for the target in
 // the plane above it (cz = -1), its own (0), below it (+1).
 template <typename T, int Q>
-__device__ __forceinline__ void flow_place(T s[4], int i, int cz, const FlowVals<T>& v, T dr, const T F[3],
+__device__ __forceinline__ void flow_place(T s[4], T own[3], int i, int cz, const FlowVals<T>& v, T dr, const T F[3],
                                            const FlowConst<T>& c) {
     const int cx = flow_px(i), cy = flow_py(i);
     if (i == 0 && cz == 0)
-        flow_own<T, Q>(s, v, dr, F, c);
+        flow_own<T, Q>(s, own, v, dr, F, c);
     else if (flow_weight<Q>((cx != 0) + (cy != 0) + (cz != 0)) != 0.0)
         flow_add<T, Q>(s, cx, cy, cz, v, c);
 }
@@ -146,7 +148,7 @@ __device__ __forceinline__ void flow_gather(const T* __restrict__ drho, const T*
                                             const T* __restrict__ F, T* __restrict__ drho_out, T* uout, long long n,
                                             int nx, int ny, int nz, int x, int y, int z, long long k,
                                             const FlowConst<T>& c) {
-    T s[4] = {T(0), T(0), T(0), T(0)};
+    T s[4] = {T(0), T(0), T(0), T(0)}, own[3] = {T(0), T(0), T(0)};
 #pragma unroll
     for (int cz = (DIM == 3 ? -1 : 0); cz <= (DIM == 3 ? 1 : 0); ++cz)
 #pragma unroll
@@ -157,13 +159,13 @@ __device__ __forceinline__ void flow_gather(const T* __restrict__ drho, const T*
                 const T uq[3] = {u[q], u[q + n], u[q + 2 * n]};
                 const T Fq[3] = {F[q], F[q + n], F[q + 2 * n]};
                 const T dr = drho[q];
-                flow_place<T, Q>(s, i, cz, flow_vals<T>(dr, uq, Fq, c), dr, Fq, c);
+                flow_place<T, Q>(s, own, i, cz, flow_vals<T>(dr, uq, Fq, c), dr, Fq, c);
             }
         }
     const T inv = T(1) / add_rn(T(1), s[0]);
     drho_out[k] = s[0];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) uout[k + a * n] = mul_rn(s[1 + a], inv);
+    for (int a = 0; a < 3; ++a) uout[k + a * n] = mul_rn(add_rn(s[1 + a], own[a]), inv);
 }
 
 // J += 3 w c x b for neighbour i of a plane.
@@ -362,7 +364,7 @@ __global__ void __launch_bounds__(kFlowThreads<T>) k_flow_march(Geo g, const T* 
     if (threadIdx.x < HALO) flow_halo<TY>(threadIdx.x, x0, y0, nx, ny, hcell, hp);
     const int z0 = blockIdx.z * chunk, z1 = min(z0 + chunk, nz);
     T cur[7], halo[7] = {};  // drho, u, F
-    T sM[4] = {}, s0[4] = {}, sP[4] = {};
+    T sM[4] = {}, s0[4] = {}, sP[4] = {}, oM[3] = {}, o0[3] = {};  // the targets' sums and own parts
     auto load = [&](int z, int q, T v[7]) {
         const int k = z * P + q;
         v[0] = drho[k];
@@ -411,16 +413,16 @@ __global__ void __launch_bounds__(kFlowThreads<T>) k_flow_march(Geo g, const T* 
                 v.M = t[7][o];
                 v.r3 = t[8][o];
             }
-            if (s > z0) flow_place<T, Q>(sM, i, 1, v, dr, Fk, c);
-            if (s >= z0 && s < z1) flow_place<T, Q>(s0, i, 0, v, dr, Fk, c);
-            if (s < z1 - 1) flow_place<T, Q>(sP, i, -1, v, dr, Fk, c);
+            if (s > z0) flow_place<T, Q>(sM, oM, i, 1, v, dr, Fk, c);
+            if (s >= z0 && s < z1) flow_place<T, Q>(s0, o0, i, 0, v, dr, Fk, c);
+            if (s < z1 - 1) flow_place<T, Q>(sP, o0, i, -1, v, dr, Fk, c);
         }
         if (s > z0 && active) {
             const int k = (s - 1) * P + p;
             const T inv = T(1) / add_rn(T(1), sM[0]);
             drho_out[k] = sM[0];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) uout[k + a * n] = mul_rn(sM[1 + a], inv);
+            for (int a = 0; a < 3; ++a) uout[k + a * n] = mul_rn(add_rn(sM[1 + a], oM[a]), inv);
         }
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
@@ -428,6 +430,8 @@ __global__ void __launch_bounds__(kFlowThreads<T>) k_flow_march(Geo g, const T* 
             s0[a] = sP[a];
             sP[a] = T(0);
         }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) oM[a] = o0[a];
         zz = zn;
     }
     if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) *tstep += 1;
