@@ -153,12 +153,10 @@ struct Launch {
                         launch_pdl(k_sweep_march_pair<float, false>, pgrid, dim3(kPairThreads), 0, st, geo(s),
                                    (const float*)bin, (float*)bout, (const float*)u, fcoef(c), chunk);
                 } else if (s.dim == 3) {
-                    if constexpr (sizeof(T) == 8) {
-                        if (s.bext_xy)
-                            k_sweep_march<T, true><<<mgrid, kMarchTX * kMarchTY, 0, st>>>(geo(s), bin, bout, u, c, chunk);
-                        else
-                            k_sweep_march<T, false><<<mgrid, kMarchTX * kMarchTY, 0, st>>>(geo(s), bin, bout, u, c, chunk);
-                    }
+                    if (s.bext_xy)
+                        k_sweep_march<T, true><<<mgrid, kMarchTX * kMarchTY, 0, st>>>(geo(s), bin, bout, u, c, chunk);
+                    else if constexpr (sizeof(T) == 8)
+                        k_sweep_march<T, false><<<mgrid, kMarchTX * kMarchTY, 0, st>>>(geo(s), bin, bout, u, c, chunk);
                 } else {
                     k_sweep_nodes<T, 2><<<grid, kNodeThreads, 0, st>>>(geo(s), bin, bout, u, c);
                 }
@@ -378,7 +376,7 @@ struct Launch {
         // at one row 24x24: 2.0 against 3.6, 36x36: 3.3 against 4.0), whose pairs an
         // odd width does without (47x46: 5.3 against 6.8); even-width slabs of
         // several planes at five rows stay with the marching sweep (60x60x304: 17.6
-        // against 16.6; at three rows 40x40x192: 7.5 against 9.5, at one row
+        // against 16.4; at three rows 40x40x192: 7.6 against 10.7, at one row
         // 24x24x300: 2.8 against 8.8).
         if (s.nx % 2 == 0 && ((G == 1 && K > 1 && s.resident) || (G > 1 && K == kSlabMaxK))) return cudaSuccess;
         // its start (tables, S) takes about 5 us longer than k_sweeps_resident's: a
@@ -511,8 +509,10 @@ struct Launch {
         return try_resident_shape<DIM, UHALO, false>(s, smem, ok);
     }
 
-    // The pair kernel serves FP32 3-D domains.
-    static bool pair_march(const State& s) { return sizeof(T) == 4 && s.dim == 3; }
+    // The pair kernel serves FP32 3-D domains, but not odd widths in an in-plane field:
+    // two scalar accesses per pair for the field too (87x86x255 32.4 us a sweep with one
+    // node per thread, 34.5 in pairs; 96x96x298, even, 47.4 and 38.5).
+    static bool pair_march(const State& s) { return sizeof(T) == 4 && s.dim == 3 && (s.nx % 2 == 0 || !s.bext_xy); }
     static SweepCoef<float> fcoef(const SweepCoef<T>& c) {
         if constexpr (sizeof(T) == 4)
             return c;
@@ -527,16 +527,14 @@ struct Launch {
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const bool pair = pair_march(s);
         if (e == cudaSuccess) {
-            if constexpr (sizeof(T) == 4)
-                e = s.bext_xy ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_march_pair<T, true>,
-                                                                              kPairThreads, 0)
-                              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_march_pair<T, false>,
-                                                                              kPairThreads, 0);
-            else
-                e = s.bext_xy ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_march<T, true>,
-                                                                              kMarchTX * kMarchTY, 0)
-                              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_march<T, false>,
-                                                                              kMarchTX * kMarchTY, 0);
+            const void* kern = (const void*)k_sweep_march<T, true>;
+            if constexpr (sizeof(T) == 4) {
+                if (pair)
+                    kern = s.bext_xy ? (const void*)k_sweep_march_pair<T, true> : (const void*)k_sweep_march_pair<T, false>;
+            } else if (!s.bext_xy) {
+                kern = (const void*)k_sweep_march<T, false>;
+            }
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, pair ? kPairThreads : kMarchTX * kMarchTY, 0);
         }
         if (e != cudaSuccess) return e;
         const int tx = pair ? 2 * kPairTXP : kMarchTX, ty = pair ? kPairTY : kMarchTY;

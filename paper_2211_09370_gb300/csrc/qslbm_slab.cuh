@@ -42,7 +42,8 @@
 //
 // Measured, us per sweep with the IB, this kernel against the route before it:
 // 24x24x96 2.0 / 3.6 (one plane per CTA, k_sweeps_resident), 24x24x300 2.8 / 8.8,
-// 40x40x192 7.5 / 9.5, 57x57x245 16.6 / 18.6 (marching sweep and IB launches),
+// 40x40x192 7.6 / 10.7, 57x57x245 16.4 / 15.9, 59x59x290 16.7 / 19.3, 61x61x150 9.4 /
+// 12.3 (marching pair sweep and IB launches),
 // 64x64x128 with an in-plane field 7.1 / 13.3.
 #pragma once
 
@@ -73,7 +74,7 @@ __host__ __device__ constexpr int slab_stride(int K) { return 2 * slab_half(K) +
 __host__ __device__ inline int slab_pairs(int nx) { return (nx + 1) / 2; }
 // Pairs between rows: padded, when the slab has room, so that the block of rows
 // K further continues the banks where a row ends (lanes of one warp cover
-// several such blocks; without, 36x36x300 took 7.3 us a sweep instead of 4.9).
+// several such blocks; without, 36x36x300 took 7.3 us a sweep, with it 5.7).
 __host__ __device__ inline int slab_row_stride(int nx, int ny, int G, int K) {
     const int XP = slab_pairs(nx);
     for (int q = XP; q < XP + 32 && G * ((ny * q + 3) / 4 * 4) <= slab_half(K) - 48; ++q)
