@@ -312,14 +312,13 @@ int qslbm_check_bounded_wait(double limit_s, int32_t counter_set, int32_t* gave_
  *    waits (a wait that times out is reported as QSLBM_ETIMEOUT by
  *    qslbm_batch_handle and the server).  Instances are admitted smallest
  *    first while their groups fit co-resident on the device;
- *  - chains (FP32): up to 16 other instances (and ones created with
- *    sweep_kernel = QSLBM_SWEEP_SPLIT) of at least 100000 nodes, the largest
- *    first, sweep each in kernels of its own, concurrently on streams of the
- *    batch's;
- *  - joint march: every remaining instance takes one persistent z-marching
- *    launch per sweep over the instances with N_mag > s, then one IB launch;
- *    the sweep's launch mode, tile shape and persistent grid are chosen by
- *    timing candidates on the batch when it is first built with such a member.
+ *  - chains (FP32): every other instance (and any created with sweep_kernel =
+ *    QSLBM_SWEEP_SPLIT), when they are at most 24, sweeps in kernels of its
+ *    own, several instances at a time on streams of the batch's;
+ *  - joint march: otherwise they take one persistent z-marching launch per
+ *    sweep over the instances with N_mag > s, then one IB launch; the sweep's
+ *    launch mode, tile shape and persistent grid are chosen by timing
+ *    candidates on the batch when it is first built with such a member.
  * Each instance follows the same arithmetic as a handle created alone with
  * QSLBM_SWEEP_SPLIT (the same expressions in the same order). */
 typedef struct qslbm_batch qslbm_batch;

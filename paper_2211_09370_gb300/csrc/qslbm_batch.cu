@@ -264,6 +264,7 @@ struct qslbm_batch {
     // chains (FP32): members [kmarch, kgroup) sweep each in a chain of its own
     // kernels, concurrently on side streams (launch_chains)
     int kgroup = 0;
+    std::vector<std::vector<int>> chain_of;  // members of each side stream
     std::vector<cudaStream_t> side;
     std::vector<cudaEvent_t> joined;
     cudaEvent_t forked = nullptr;
@@ -456,21 +457,27 @@ void launch_groups(qslbm_batch& B, cudaStream_t st) {
     }
 }
 
-// A marching member of an FP32 batch in a chain of its own kernels: the pair sweep on
-// a grid of one wave and its IB pass, which run concurrently with the other chains.
-// Both kernels are bound by latency (the sweep issues in 39 % of the cycles), so
-// that members' kernels fill each other's stalls, tails and launch gaps; in the joint
-// march every sweep waits for the whole batch twice, and tiles of one row a thread
-// cost more.  Us a sweep, joint / chains: eight pipes of 32x32x183 to 85x85x505 186 /
-// 146; one 96x96x512 67.7 / 51.6, three 88x88x300 108 / 75, four 72x72x200 79.5 /
-// 54.9, six 48x48x180 49.0 / 36.1, eight 40x40x130 39.0 / 30.1, nine 32x32x100 19.8 /
-// 12.3; nothing smaller was measured.  At most kChains of them, the largest, with a
-// stream each (a graph of a step holds 2 N_mag nodes per chain).
-constexpr int kChains = 16;
-constexpr long long kChainNodes = 100000;
+// Chains: the marching members of an FP32 batch, each in kernels of its own (the pair
+// sweep on a grid of one wave and its IB pass), several members at a time.  Both
+// kernels are bound by latency (the sweep issues in 39 % of the cycles), so that
+// members' kernels fill each other's stalls, tails and launch gaps; in the joint march
+// every sweep waits for the whole batch twice, and tiles of one row a thread cost
+// more.  All marching members or none, of at most kChains: 64 uneven pipes take 378 ms
+// a step jointly, 526 in chains (a graph of 29 000 kernels), 551 in 16 chains beside a
+// joint march of the rest.
+//
+// Streams: as many as keep kChainInFlight nodes in flight.  Members above L2 gain from
+// the second and third only, small ones from every one.  Ms a step (270 sweeps), joint
+// / one, two, three, six, sixteen streams: eight pipes of 32x32x183 to 85x85x505 49.3 /
+// 45.6, 38.4, 39.6, 39.6, 39.6; 24 of the same range 136 / 144, 114, 113, 114, 116; six
+// 48x48x180 12.7 / 18.3, 9.9, 8.9, 9.1, 9.1; nine 32x32x100 5.0 / 22.7, 13.6, 8.2, 5.5,
+// 3.0 (nine).
+constexpr int kChains = 24;
+constexpr int kChainStreams = 16;
+constexpr long long kChainInFlight = 1200000;
 
 bool chain_member(const State& s) {
-    return s.esz == 4 && s.dim == 3 && s.n >= kChainNodes && (s.ib.nm == 0 || s.ib_staged_smem > 0);
+    return s.esz == 4 && s.dim == 3 && (s.ib.nm == 0 || s.ib_staged_smem > 0);
 }
 
 void launch_chain(qslbm_batch& B, int k, cudaStream_t st) {
@@ -497,7 +504,27 @@ void launch_chain(qslbm_batch& B, int k, cudaStream_t st) {
 
 // Streams and shared-memory limits for the chains of the members [kmarch, kgroup).
 int prepare_chains(qslbm_batch& B) {
-    const size_t n = (size_t)(B.kgroup - B.kmarch);
+    const int nc = B.kgroup - B.kmarch;
+    long long nodes = 0;
+    for (int k = B.kmarch; k < B.kgroup; ++k) nodes += qslbm::handle_state_mut(B.members[k]).n;
+    size_t n = 0;
+    if (nc > 0)
+        n = (size_t)std::min<long long>(nc, std::clamp<long long>(kChainInFlight * nc / nodes, 3, kChainStreams));
+    B.chain_of.assign(n, {});
+    // the longest chain left to the stream with the least work so far
+    auto work = [&](int k) {
+        const State& s = qslbm::handle_state_mut(B.members[k]);
+        return s.n * (long long)s.units.n_mag;
+    };
+    std::vector<int> order(B.kgroup - B.kmarch);
+    std::iota(order.begin(), order.end(), B.kmarch);
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return work(a) > work(b); });
+    std::vector<long long> load(n, 0);
+    for (int k : order) {
+        const size_t j = std::min_element(load.begin(), load.end()) - load.begin();
+        B.chain_of[j].push_back(k);
+        load[j] += work(k);
+    }
     if (n > 0 && !B.forked) BCHK(cudaEventCreateWithFlags(&B.forked, cudaEventDisableTiming));
     while (B.side.size() < n) {
         cudaStream_t st = nullptr;
@@ -521,16 +548,16 @@ int prepare_chains(qslbm_batch& B) {
 template <typename T>
 void launch_step(qslbm_batch& B, cudaStream_t st) {
     launch_groups<T>(B, st);
-    // the chains beside the joint sweeps of the other marching members
-    const int nc = B.kgroup - B.kmarch;
-    if (nc > 0) cudaEventRecord(B.forked, st);
-    for (int j = 0; j < nc; ++j) {
+    // the chains, or the joint sweeps of the marching members
+    const int ns = (int)B.chain_of.size();
+    if (ns > 0) cudaEventRecord(B.forked, st);
+    for (int j = 0; j < ns; ++j) {
         cudaStreamWaitEvent(B.side[j], B.forked, 0);
-        launch_chain(B, B.kmarch + j, B.side[j]);
+        for (int k : B.chain_of[j]) launch_chain(B, k, B.side[j]);
         cudaEventRecord(B.joined[j], B.side[j]);
     }
     for (int s = 0; s < B.max_nmag; ++s) launch_sweep<T>(B, s, B.threads, B.grid, st);
-    for (int j = 0; j < nc; ++j) cudaStreamWaitEvent(st, B.joined[j], 0);  // (an error ends the graph capture)
+    for (int j = 0; j < ns; ++j) cudaStreamWaitEvent(st, B.joined[j], 0);  // (an error ends the graph capture)
     const int K = (int)B.members.size();
     auto* d = (qslbm::InstDesc<T>*)B.desc;
     qslbm::k_batch_force<T><<<B.h_pfirst[K], qslbm::kNodeThreads, 0, st>>>(d, B.pfirst, K);
@@ -987,22 +1014,19 @@ int set_members(qslbm_batch* B, const std::vector<qslbm_handle*>& hs, const std:
         for (int i : adm) spread[i] = planes_at(i, lo);
         for (int i : adm) gp[i] = spread[i];
     }
-    // chains: the marching members of some size (FP32), the largest first
-    std::vector<char> chain(count, 0);
-    if (B->precision == QSLBM_FP32) {
-        std::vector<int> big;
-        for (int i = 0; i < count; ++i)
-            if (gp[i] == 0 && chain_member(qslbm::handle_state_mut(hs[i]))) big.push_back(i);
-        std::stable_sort(big.begin(), big.end(), [&](int a, int b) {
-            return qslbm::handle_state_mut(hs[a]).n > qslbm::handle_state_mut(hs[b]).n;
-        });
-        if (big.size() > kChains) big.resize(kChains);
-        for (int i : big) chain[i] = 1;
-    }
+    // chains or the joint march, for all marching members alike
+    int marching = 0;
+    bool chains = B->precision == QSLBM_FP32;
+    for (int i = 0; i < count; ++i)
+        if (gp[i] == 0) {
+            ++marching;
+            chains = chains && chain_member(qslbm::handle_state_mut(hs[i]));
+        }
+    chains = chains && marching <= kChains;
     std::vector<int> idx(count);
     std::iota(idx.begin(), idx.end(), 0);
     // jointly marching members first, then the chains', then the groups'
-    auto kind = [&](int i) { return gp[i] > 0 ? 2 : (chain[i] ? 1 : 0); };
+    auto kind = [&](int i) { return gp[i] > 0 ? 2 : (chains ? 1 : 0); };
     std::stable_sort(idx.begin(), idx.end(), [&](int a, int b) {
         if (kind(a) != kind(b)) return kind(a) < kind(b);
         return qslbm::handle_state_mut(hs[a]).units.n_mag > qslbm::handle_state_mut(hs[b]).units.n_mag;

@@ -1,7 +1,7 @@
-"""Large members of an FP32 batch, which sweep in chains of their own kernels beside
-the joint sweeps and the resident groups of the others: every member as on its own
-handle (same roundings, so to the bit), with different sweep counts, an in-plane
-field, several steps per graph, and as long as a chunk of steps and a rest."""
+"""FP32 batch members off the resident groups sweep in chains of their own kernels, or
+jointly when there are more than 24: every member as on its own handle (same
+roundings, so to the bit), with different sweep counts, an in-plane field, members
+that share a stream, and resident groups beside them."""
 import numpy as np
 import pytest
 
@@ -19,7 +19,7 @@ OTHERS = {
     "alone": [],
     "with_a_field": [dict(nx=90, ny=90, nz=52, diameter=80.0, n_mag=4, b0_kind="field", seed=74)],
     "with_groups": [dict(nx=24, ny=24, nz=40, diameter=16.0, n_mag=5, seed=75)],
-    "with_joint_sweeps": [dict(nx=40, ny=40, nz=20, diameter=30.0, n_mag=8, sweep_kernel="split", seed=76),
+    "with_small_ones": [dict(nx=40, ny=40, nz=20, diameter=30.0, n_mag=8, sweep_kernel="split", seed=76),
                           dict(nx=33, ny=35, nz=12, diameter=24.0, n_mag=3, sweep_kernel="split", seed=77)],
 }
 
@@ -39,6 +39,24 @@ def test_chains_match_single_handles(others):
     for i, p in enumerate(ps):
         with Solver(dict(p, sweep_kernel="split")) as s:
             s.step(steps)
+            want = s.state()
+        for a, b in zip(got[i], want):
+            np.testing.assert_array_equal(a, b, err_msg=str(i))
+
+
+@pytest.mark.parametrize("count", [20, 24, 25])
+def test_many_marching_members(count):
+    # more members than streams; as many as take chains; one more, which march jointly
+    ps = [W.small_pipe(nx=12 + i % 3, ny=11, nz=3 + i % 4, diameter=7.0, n_mag=2 + i % 5, Ha=20.0, Rm=2e-3, seed=i,
+                       sweep_kernel="split") for i in range(count)]
+    with Batch(ps) as B:
+        chains = sum(2 * p["n_mag"] for p in ps)
+        assert (B.info()["launches_per_step"] == chains + 3) == (count <= 24)
+        B.step(3)
+        got = [B.member(i).state() for i in range(count)]
+    for i in (0, 7, count - 1):
+        with Solver(ps[i]) as s:
+            s.step(3)
             want = s.state()
         for a, b in zip(got[i], want):
             np.testing.assert_array_equal(a, b, err_msg=str(i))
