@@ -141,7 +141,8 @@ def replica_throughput(world: int, nodes_per_rank: int, steps: int, slowest_ms: 
     return world * nodes_per_rank * steps / (slowest_ms / 1e3) / 1e6
 
 
-KERNEL_SOURCES = ("qslbm_kernels.cuh", "qslbm_resident.cuh", "qslbm_slab.cuh", "qslbm_fused.cuh", "qslbm_launch.cuh")
+KERNEL_SOURCES = ("qslbm_kernels.cuh", "qslbm_flow.cuh", "qslbm_resident.cuh", "qslbm_resident64.cuh",
+                  "qslbm_slab.cuh", "qslbm_fused.cuh", "qslbm_launch.cuh")
 
 
 def kernel_source_sha() -> str:
@@ -171,17 +172,19 @@ def profiled_traffic(workload: str, kernel: str):
 def sweep_kernel_info(solver, p):
     """(launches per flow step: the sweeps', force, flow and the IB on u; kernel
     description; sweeps per launch) of the handle's magnetic sub-iteration kernel."""
-    k = solver.units["sweep_kernel"]
+    plan = solver.plan()
+    k = plan["kernel"]
+    t = f"{k}<{p.get('precision', 'fp32')}>"
     n_mag = solver.units["n_mag"]
-    if k == "resident":
-        return 4, "k_sweeps_resident<float,3> (all sweeps + IB on b, planes held in shared memory)", n_mag
-    if k == "fused":
-        return n_mag + 3, ("k_sweep_fused<float> (one sweep + IB on b: each CTA marches a band of rows of a z "
+    if k.startswith("k_sweeps_"):
+        return 4, f"{t} (all sweeps + IB on b in shared memory, {plan['planes']} plane(s) a CTA)", n_mag
+    if k == "k_sweep_fused":
+        return n_mag + 3, (f"{t} (one sweep + IB on b: each CTA marches a band of rows of a z "
                            "chunk, staged by TMA, and corrects it in shared memory)"), 1
-    if k == "split":
-        return 2 * n_mag + 3, ("k_sweep_march_pair<float> + k_ib_staged<float> (one sweep: z-marching stencil, "
-                               "then the IB corrector on b, one CTA per plane)"), 1
-    return n_mag + 3, "k_sweep_ib<float,3> (one sweep + IB on b, one z plane per CTA)", 1
+    if k == "k_sweep_ib":
+        return n_mag + 3, f"{t} (one sweep + IB on b, one z plane per CTA)", 1
+    return 2 * n_mag + 3, (f"{t} + k_ib_staged (one sweep: z-marching stencil, "
+                           "then the IB corrector on b, one CTA per plane)"), 1
 
 
 def roofline_block(solver, p, workload, sweep_ms, peak, peak_kind):

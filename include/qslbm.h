@@ -212,6 +212,28 @@ int qslbm_create(const qslbm_params* p, qslbm_handle** out);
 /* Lattice-unit values of the handle.  Errors: QSLBM_EINVAL (NULL argument). */
 int qslbm_get_units(const qslbm_handle* h, qslbm_units* out);
 
+/* The kernel that runs a handle's magnetic sweeps, and its shape.
+ *   kernel   QSLBM_KERNEL_*
+ *   ctas     CTAs of a launch
+ *   threads  threads per CTA
+ *   rows     SLAB, MARCH_PAIR: rows per thread; CLUSTER64: rows per CTA;
+ *            FUSED: rows per band; else 0
+ *   planes   z planes per CTA, at most */
+#define QSLBM_KERNEL_PLANES 1     /* k_sweep_ib: one sweep and its IB per launch, a plane per CTA */
+#define QSLBM_KERNEL_RESIDENT 2   /* k_sweeps_resident: all sweeps, a plane per CTA */
+#define QSLBM_KERNEL_SLAB 3       /* k_sweeps_slab: all sweeps (FP32), planes per CTA as needed */
+#define QSLBM_KERNEL_RESIDENT64 4 /* k_sweeps_resident64: all sweeps (FP64), a plane per CTA */
+#define QSLBM_KERNEL_CLUSTER64 5  /* k_sweeps_cluster64: all sweeps (FP64, 2-D), one cluster */
+#define QSLBM_KERNEL_FUSED 6      /* k_sweep_fused: one sweep and its IB per launch */
+#define QSLBM_KERNEL_MARCH_PAIR 7 /* k_sweep_march_pair (FP32), then the IB */
+#define QSLBM_KERNEL_MARCH 8      /* k_sweep_march, then the IB */
+#define QSLBM_KERNEL_NODES 9      /* k_sweep_nodes (2-D), then the IB */
+typedef struct qslbm_sweep_plan_t {
+    int32_t kernel, ctas, threads, rows, planes;
+} qslbm_sweep_plan_t;
+/* Errors: QSLBM_EINVAL (NULL argument). */
+int qslbm_sweep_plan(const qslbm_handle* h, qslbm_sweep_plan_t* out);
+
 /* Queue nsteps >= 0 flow steps (N_mag sweeps + IB on b each, force, flow
  * update, IB on u).  Asynchronous.  Errors: QSLBM_EINVAL, QSLBM_ECUDA. */
 int qslbm_step(qslbm_handle* h, int64_t nsteps);

@@ -53,6 +53,15 @@ class qslbm_units(C.Structure):
                 ("sweep_us_fused", C.c_double), ("sweep_us_split", C.c_double)]
 
 
+class qslbm_sweep_plan_t(C.Structure):
+    _fields_ = [(k, C.c_int32) for k in ("kernel", "ctas", "threads", "rows", "planes")]
+
+
+SWEEP_PLAN_KERNEL = {1: "k_sweep_ib", 2: "k_sweeps_resident", 3: "k_sweeps_slab", 4: "k_sweeps_resident64",
+                     5: "k_sweeps_cluster64", 6: "k_sweep_fused", 7: "k_sweep_march_pair", 8: "k_sweep_march",
+                     9: "k_sweep_nodes"}
+
+
 class qslbm_obs(C.Structure):
     _fields_ = [("step", C.c_int64)] + [(k, C.c_double) for k in (
         "mass", "mass_drift", "E_k", "E_m", "pump", "visc", "joule", "qs_residual", "steady_residual")] + [
@@ -88,8 +97,8 @@ class qslbm_server_stats_t(C.Structure):
 
 
 # every symbol the header declares (checked by the CPU test-suite)
-EXPORTS = ("qslbm_params_init", "qslbm_create", "qslbm_get_units", "qslbm_step", "qslbm_mag_sweeps",
-           "qslbm_observables", "qslbm_get_state", "qslbm_set_state", "qslbm_step_host", "qslbm_sync",
+EXPORTS = ("qslbm_params_init", "qslbm_create", "qslbm_get_units", "qslbm_sweep_plan", "qslbm_step",
+           "qslbm_mag_sweeps", "qslbm_observables", "qslbm_get_state", "qslbm_set_state", "qslbm_step_host", "qslbm_sync",
            "qslbm_destroy", "qslbm_strerror", "qslbm_last_error", "qslbm_observables_static",
            "qslbm_check_bounded_wait",
            "qslbm_batch_create", "qslbm_batch_step", "qslbm_batch_handle", "qslbm_batch_info",
@@ -113,6 +122,7 @@ def load(path: str | None = None):
     L.qslbm_params_init.restype = None
     L.qslbm_create.argtypes = [C.POINTER(qslbm_params), C.POINTER(hp)]
     L.qslbm_get_units.argtypes = [hp, C.POINTER(qslbm_units)]
+    L.qslbm_sweep_plan.argtypes = [hp, C.POINTER(qslbm_sweep_plan_t)]
     L.qslbm_step.argtypes = [hp, C.c_int64]
     L.qslbm_mag_sweeps.argtypes = [hp, C.c_int32]
     L.qslbm_observables.argtypes = [hp, C.POINTER(qslbm_obs), dp, dp, dp]
@@ -150,7 +160,7 @@ def load(path: str | None = None):
         getattr(L, name).restype = C.c_int
     L.qslbm_last_error.argtypes = []
     L.qslbm_last_error.restype = C.c_char_p
-    for name in ("qslbm_create", "qslbm_get_units", "qslbm_step", "qslbm_mag_sweeps", "qslbm_observables",
+    for name in ("qslbm_create", "qslbm_get_units", "qslbm_sweep_plan", "qslbm_step", "qslbm_mag_sweeps", "qslbm_observables",
                  "qslbm_get_state", "qslbm_set_state", "qslbm_step_host", "qslbm_sync", "qslbm_destroy"):
         getattr(L, name).restype = C.c_int
     _lib = L
@@ -274,6 +284,14 @@ class Solver:
 
     def __exit__(self, *a):
         self.close()
+
+    def plan(self) -> dict:
+        """The kernel that runs this handle's sweeps and its shape (qslbm_sweep_plan)."""
+        p = qslbm_sweep_plan_t()
+        check(self.L.qslbm_sweep_plan(self.h, C.byref(p)), "qslbm_sweep_plan")
+        d = {k: getattr(p, k) for k, _ in p._fields_}
+        d["kernel"] = SWEEP_PLAN_KERNEL[p.kernel]
+        return d
 
     def step(self, n: int = 1):
         check(self.L.qslbm_step(self.h, int(n)), "qslbm_step")

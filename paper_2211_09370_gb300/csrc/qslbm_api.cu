@@ -1038,6 +1038,13 @@ int qslbm_get_units(const qslbm_handle* h, qslbm_units* out) {
     return QSLBM_OK;
 }
 
+int qslbm_sweep_plan(const qslbm_handle* h, qslbm_sweep_plan_t* out) {
+    if (!h || !out) return bad_argument("qslbm_sweep_plan: NULL argument");
+    std::memset(out, 0, sizeof(*out));
+    ops(h->s).sweep_plan(h->s, out);
+    return QSLBM_OK;
+}
+
 int qslbm_step(qslbm_handle* h, int64_t nsteps) {
     if (!h) return bad_argument("qslbm_step: NULL handle");
     return step_impl(h->s, nsteps);

@@ -114,6 +114,7 @@ struct State {
     bool resident = false;
     bool launch_error = false;  // a cudaLaunchKernelEx call failed
     int march_chunk = 16;       // z planes per CTA of the marching sweep (one wave)
+    int march_rows = 0;         // rows per thread of the FP32 pair sweep (0: one node per thread)
     size_t ib_staged_smem = 0;  // shared memory of k_ib_staged, 0 when it does not fit
     int ib_staged_u = 1;        // its shell nodes per thread per batch of loads (1, 2, 4 or 5)
     bool resident_uhalo = false;
@@ -183,6 +184,7 @@ struct Ops {
     // (no allocation)
     cudaError_t (*plan_resident)(State&);
     cudaError_t (*plan_march)(State&);  // sets s.march_chunk and s.ib_staged_smem
+    void (*sweep_plan)(const State&, qslbm_sweep_plan_t*);  // the sweep kernel and its shape
     // launch shape of the fused sweep for the tables already in s (fu_TY,
     // fu_bands, fu_smem): sets fu_threads, fu_chunk, fu_chunks, or clears
     // s.fused when it cannot run here

@@ -513,6 +513,31 @@ struct Launch {
     // two scalar accesses per pair for the field too (87x86x255 32.4 us a sweep with one
     // node per thread, 34.5 in pairs; 96x96x298, even, 47.4 and 38.5).
     static bool pair_march(const State& s) { return sizeof(T) == 4 && s.dim == 3 && (s.nx % 2 == 0 || !s.bext_xy); }
+    static void sweep_plan(const State& s, qslbm_sweep_plan_t* out) {
+        if (s.resident && s.slab_ctas > 0)
+            *out = {QSLBM_KERNEL_SLAB, s.slab_ctas, s.slab_threads, s.slab_rows,
+                    (s.nz + s.slab_ctas - 1) / s.slab_ctas};
+        else if (s.resident && s.c2_ctas > 0)
+            *out = {QSLBM_KERNEL_CLUSTER64, s.c2_ctas, kC2Threads, s.c2_rows, 1};
+        else if (s.resident && sizeof(T) == 8 && s.dim == 3)
+            *out = {QSLBM_KERNEL_RESIDENT64, s.nz, kRes64Threads, 0, 1};
+        else if (s.resident)
+            *out = {QSLBM_KERNEL_RESIDENT, s.nz,
+                    small_plane(s) ? ResidentShape<T, true>::threads : ResidentShape<T, false>::threads, 0, 1};
+        else if (s.fused)
+            *out = {QSLBM_KERNEL_FUSED, s.fu_bands * s.fu_chunks, s.fu_threads, s.fu_TY, s.fu_chunk};
+        else if (s.p.sweep_kernel != QSLBM_SWEEP_SPLIT)
+            *out = {QSLBM_KERNEL_PLANES, s.nz, kPlaneThreads, 0, 1};
+        else if (s.dim == 2)
+            *out = {QSLBM_KERNEL_NODES, (s.nx * s.ny + kNodeThreads - 1) / kNodeThreads, kNodeThreads, 0, 1};
+        else {
+            const bool pair = s.march_rows > 0;
+            const int tx = pair ? 2 * kPairTXP : kMarchTX, ty = pair ? kPairTY : kMarchTY;
+            *out = {pair ? QSLBM_KERNEL_MARCH_PAIR : QSLBM_KERNEL_MARCH,
+                    ((s.nx + tx - 1) / tx) * ((s.ny + ty - 1) / ty) * ((s.nz + s.march_chunk - 1) / s.march_chunk),
+                    pair ? kPairThreads : kMarchTX * kMarchTY, s.march_rows, s.march_chunk};
+        }
+    }
     static SweepCoef<float> fcoef(const SweepCoef<T>& c) {
         if constexpr (sizeof(T) == 4)
             return c;
@@ -544,6 +569,7 @@ struct Launch {
         long long chunk = (s.nz + per_column - 1) / per_column;
         chunk = std::max<long long>(chunk, 4);  // keep the z halo overhead small
         s.march_chunk = (int)std::min<long long>(chunk, s.nz);
+        s.march_rows = pair ? 2 : 0;
         // the staged IB corrector, when the plane's shell fits shared memory
         // and the shell nodes' marker lists are padded
         s.ib_staged_smem = 0;
@@ -819,8 +845,8 @@ struct Launch {
 
     static const Ops& table() {
         static const Ops o = {&init,     &sweeps,        &force_flow, &observe,     &observe_fields,
-                              &to_f64,   &from_f64,      &plan_resident, &plan_march, &plan_fused,
-                              &tune_fused};
+                              &to_f64,   &from_f64,      &plan_resident, &plan_march, &sweep_plan,
+                              &plan_fused, &tune_fused};
         return o;
     }
 };
