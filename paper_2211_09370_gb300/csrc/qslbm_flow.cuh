@@ -266,6 +266,20 @@ constexpr int kFlowTY = sizeof(T) == 4 ? 8 : 4;  // (the staged planes fit stati
 template <typename T>
 constexpr int kFlowThreads = kFlowTX * kFlowTY<T>;
 
+// The tile and z chunk of this CTA: one grid dimension counts them all (tiles along x,
+// then y, then chunks), since the other two hold 65535 CTAs and a long thin domain has
+// more rows or planes than that many tiles.
+struct FlowTile {
+    int x0, y0, z0, z1;
+};
+template <typename T>
+__device__ __forceinline__ FlowTile flow_tile(int nx, int ny, int nz, int chunk) {
+    const unsigned tx = (unsigned)(nx + kFlowTX - 1) / kFlowTX, ty = (unsigned)(ny + kFlowTY<T> - 1) / kFlowTY<T>;
+    const unsigned row = blockIdx.x / tx, layer = row / ty;
+    const int z0 = (int)layer * chunk;
+    return {(int)(blockIdx.x - row * tx) * kFlowTX, (int)(row - layer * ty) * kFlowTY<T>, z0, min(z0 + chunk, nz)};
+}
+
 // Halo cell h of a tile: rows above and below (with the corners), columns left and
 // right.  cell: its offset in a staged plane; node: in-plane index (periodic image).
 template <int TY>
@@ -294,13 +308,13 @@ __global__ void __launch_bounds__(kFlowThreads<T>) k_force_march(Geo g, const T*
     const int nx = g.nx, ny = g.ny, nz = g.nz, P = nx * ny;
     const int n = (int)g.n;
     const int tx = threadIdx.x % kFlowTX, ty = threadIdx.x / kFlowTX;
-    const int x0 = blockIdx.x * kFlowTX, y0 = blockIdx.y * TY, x = x0 + tx, y = y0 + ty;
+    const FlowTile ft = flow_tile<T>(nx, ny, nz, chunk);
+    const int x0 = ft.x0, y0 = ft.y0, z0 = ft.z0, z1 = ft.z1, x = x0 + tx, y = y0 + ty;
     const bool active = x < nx && y < ny;
     const int p = (y % ny) * nx + x % nx;
     const int cell = (ty + 1) * W + tx + 1;
     int hcell = -1, hp = 0;
     if (threadIdx.x < HALO) flow_halo<TY>(threadIdx.x, x0, y0, nx, ny, hcell, hp);
-    const int z0 = blockIdx.z * chunk, z1 = min(z0 + chunk, nz);
     const T fb = body_force_at(c, *tstep);
     T cur[3], halo[3] = {}, last[3] = {};
     T Jm[3] = {}, J0[3] = {}, Jp[3] = {};
@@ -356,13 +370,13 @@ __global__ void __launch_bounds__(kFlowThreads<T>) k_flow_march(Geo g, const T* 
     const int n = (int)g.n;
     const FlowConst<T> c(fc);
     const int tx = threadIdx.x % kFlowTX, ty = threadIdx.x / kFlowTX;
-    const int x0 = blockIdx.x * kFlowTX, y0 = blockIdx.y * TY, x = x0 + tx, y = y0 + ty;
+    const FlowTile ft = flow_tile<T>(nx, ny, nz, chunk);
+    const int x0 = ft.x0, y0 = ft.y0, z0 = ft.z0, z1 = ft.z1, x = x0 + tx, y = y0 + ty;
     const bool active = x < nx && y < ny;
     const int p = (y % ny) * nx + x % nx;
     const int cell = (ty + 1) * W + tx + 1;
     int hcell = -1, hp = 0;
     if (threadIdx.x < HALO) flow_halo<TY>(threadIdx.x, x0, y0, nx, ny, hcell, hp);
-    const int z0 = blockIdx.z * chunk, z1 = min(z0 + chunk, nz);
     T cur[7], halo[7] = {};  // drho, u, F
     T sM[4] = {}, s0[4] = {}, sP[4] = {}, oM[3] = {}, o0[3] = {};  // the targets' sums and own parts
     auto load = [&](int z, int q, T v[7]) {
@@ -434,7 +448,7 @@ __global__ void __launch_bounds__(kFlowThreads<T>) k_flow_march(Geo g, const T* 
         for (int a = 0; a < 3; ++a) oM[a] = o0[a];
         zz = zn;
     }
-    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) *tstep += 1;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *tstep += 1;
 }
 
 }  // namespace qslbm

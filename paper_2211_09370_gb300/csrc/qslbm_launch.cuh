@@ -777,8 +777,9 @@ struct Launch {
             k_flow_nodes<T, 9><<<blocks, kFlowNodeThreads, 0, st>>>(geo(s), dr, u, F, dro, uo, c, s.tdev);
         } else {
             const int chunk = flow_chunk(s);
-            const dim3 grid((unsigned)((s.nx + kFlowTX - 1) / kFlowTX),
-                            (unsigned)((s.ny + kFlowTY<T> - 1) / kFlowTY<T>), (unsigned)((s.nz + chunk - 1) / chunk));
+            const unsigned grid = (unsigned)((s.nx + kFlowTX - 1) / kFlowTX) *
+                                  (unsigned)((s.ny + kFlowTY<T> - 1) / kFlowTY<T>) *
+                                  (unsigned)((s.nz + chunk - 1) / chunk);
             constexpr int threads = kFlowThreads<T>;
             if (s.units.flow_q == 27) {
                 k_force_march<T, 27><<<grid, threads, 0, st>>>(geo(s), b, F, fc, s.tdev, chunk);
