@@ -134,15 +134,15 @@ __global__ void __launch_bounds__(kNodeThreads, (kIbStagedMinBlocks<T, U>)) k_ba
 // Sweep s of one member alone, on node pairs, and its IB pass: the two kernels of its
 // chain (launch_chain).  D: the member, of which the parities are
 // read where they advance (live).
-template <bool XY>
-__global__ void __launch_bounds__(kPairThreads, 3) k_chain_sweep(InstDesc<float> D, const InstDesc<float>* live,
-                                                                 int s, int chunk) {
-    __shared__ __align__(16) PairTile tile;
+template <bool XY, int R>
+__global__ void __launch_bounds__(kPairThreads, kPairMinBlocks<R>)
+    k_chain_sweep(InstDesc<float> D, const InstDesc<float>* live, int s, int chunk) {
+    __shared__ __align__(16) PairTile<R> tile;
     pdl_trigger();
     pdl_wait();
     const int par = (live->bpar + s) & 1;
     const float* u = live->fpar ? D.u[1] : D.u[0];
-    pair_tile<XY>(D.g, par ? D.b[1] : D.b[0], par ? D.b[0] : D.b[1], u, D.sc, blockIdx.x, blockIdx.y, blockIdx.z, chunk, tile);
+    pair_tile<XY, R>(D.g, par ? D.b[1] : D.b[0], par ? D.b[0] : D.b[1], u, D.sc, blockIdx.x, blockIdx.y, blockIdx.z, chunk, tile);
 }
 template <int U>
 __global__ void __launch_bounds__(kNodeThreads, (kIbStagedMinBlocks<float, U>))
@@ -265,6 +265,7 @@ struct qslbm_batch {
     // kernels, concurrently on side streams (launch_chains)
     int kgroup = 0;
     std::vector<std::vector<int>> chain_of;  // members of each side stream
+    std::vector<std::pair<int, int>> chain_shape;  // per member: rows per thread, planes per CTA of its sweep
     std::vector<cudaStream_t> side;
     std::vector<cudaEvent_t> joined;
     cudaEvent_t forked = nullptr;
@@ -471,7 +472,8 @@ void launch_groups(qslbm_batch& B, cudaStream_t st) {
 // / one, two, three, six, sixteen streams: eight pipes of 32x32x183 to 85x85x505 49.3 /
 // 45.6, 38.4, 39.6, 39.6, 39.6; 24 of the same range 136 / 144, 114, 113, 114, 116; six
 // 48x48x180 12.7 / 18.3, 9.9, 8.9, 9.1, 9.1; nine 32x32x100 5.0 / 22.7, 13.6, 8.2, 5.5,
-// 3.0 (nine).
+// 3.0 (nine).  One to three members, joint / chains: one 32x32x100 2.12 / 1.46, two 2.28 /
+// 1.91, three 2.88 / 1.85, one 40x40x192 3.02 / 2.34, two 48x48x180 5.23 / 3.32.
 constexpr int kChains = 24;
 constexpr int kChainStreams = 16;
 constexpr long long kChainInFlight = 1200000;
@@ -484,15 +486,18 @@ void launch_chain(qslbm_batch& B, int k, cudaStream_t st) {
     const State& s = qslbm::handle_state_mut(B.members[k]);
     const auto* live = (const qslbm::InstDesc<float>*)B.desc + k;
     const qslbm::InstDesc<float> D = make_desc<float>(s);
+    const auto [rows, chunk] = B.chain_shape[k];
+    const bool one = rows == 1;
+    const int ty = one ? qslbm::kPairTY<1> : qslbm::kPairTY<2>;
     const dim3 grid((unsigned)((s.nx + 2 * qslbm::kPairTXP - 1) / (2 * qslbm::kPairTXP)),
-                    (unsigned)((s.ny + qslbm::kPairTY - 1) / qslbm::kPairTY),
-                    (unsigned)((s.nz + s.march_chunk - 1) / s.march_chunk));
+                    (unsigned)((s.ny + ty - 1) / ty), (unsigned)((s.nz + chunk - 1) / chunk));
+    const auto sweep = s.bext_xy ? (one ? qslbm::k_chain_sweep<true, 1> : qslbm::k_chain_sweep<true, 2>)
+                                 : (one ? qslbm::k_chain_sweep<false, 1> : qslbm::k_chain_sweep<false, 2>);
     const int R = s.ib.max_ring, S = s.ib.max_shell;
     const dim3 ig((unsigned)s.nz), ib(qslbm::kNodeThreads);
     for (int i = 0; i < s.units.n_mag; ++i) {
         // (the first waits for the kernels before the step's sweeps in full)
-        launch_pdl(i > 0, s.bext_xy ? qslbm::k_chain_sweep<true> : qslbm::k_chain_sweep<false>, grid,
-                   dim3(qslbm::kPairThreads), 0, st, D, live, i, s.march_chunk);
+        launch_pdl(i > 0, sweep, grid, dim3(qslbm::kPairThreads), 0, st, D, live, i, chunk);
         if (s.ib.nm == 0) continue;
         const auto kern = s.ib_staged_u == 1   ? qslbm::k_chain_ib<1>
                           : s.ib_staged_u == 2 ? qslbm::k_chain_ib<2>
@@ -511,6 +516,12 @@ int prepare_chains(qslbm_batch& B) {
     if (nc > 0)
         n = (size_t)std::min<long long>(nc, std::clamp<long long>(kChainInFlight * nc / nodes, 3, kChainStreams));
     B.chain_of.assign(n, {});
+    // each sweep's grid for its part of the device: as many run at a time as there are
+    // streams (two 48x48x180: 3320 us a step, 3530 with grids that each fill the device)
+    B.chain_shape.assign(B.members.size(), {2, 1});
+    for (int k = B.kmarch; k < B.kgroup; ++k)
+        BCHK(qslbm::ops_f32().pair_shape(qslbm::handle_state_mut(B.members[k]), (int)n, &B.chain_shape[k].first,
+                                         &B.chain_shape[k].second));
     // the longest chain left to the stream with the least work so far
     auto work = [&](int k) {
         const State& s = qslbm::handle_state_mut(B.members[k]);

@@ -183,7 +183,10 @@ struct Ops {
     // s.resident, s.resident_uhalo, s.resident_smem and the kernel's own shape
     // (no allocation)
     cudaError_t (*plan_resident)(State&);
-    cudaError_t (*plan_march)(State&);  // sets s.march_chunk and s.ib_staged_smem
+    cudaError_t (*plan_march)(State&);  // sets s.march_chunk, s.march_rows and s.ib_staged_smem
+    // rows per thread and z planes per CTA of the FP32 pair sweep on a domain that
+    // shares the device with share - 1 others
+    cudaError_t (*pair_shape)(const State&, int share, int* rows, int* chunk);
     void (*sweep_plan)(const State&, qslbm_sweep_plan_t*);  // the sweep kernel and its shape
     // launch shape of the fused sweep for the tables already in s (fu_TY,
     // fu_bands, fu_smem): sets fu_threads, fu_chunk, fu_chunks, or clears

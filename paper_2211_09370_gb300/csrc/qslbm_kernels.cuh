@@ -492,8 +492,8 @@ __global__ void __launch_bounds__(kMarchTX* kMarchTY) k_sweep_march(Geo g, const
 }
 
 // FP32 z-marching sweep on x-adjacent node pairs: a CTA of 128 threads owns a
-// tile of 32 x 16 nodes and walks a chunk of z planes; a thread owns a node pair
-// in each of two rows.  EMF form as in march_tile, in packed arithmetic (one
+// tile of 32 x 8 R nodes and walks a chunk of z planes; a thread owns a node pair
+// in each of R rows, two on large domains, one on small ones.  EMF form as in march_tile, in packed arithmetic (one
 // instruction for a pair, the same roundings).  The staged plane is
 // double-buffered (one barrier per plane) and every global load is issued one
 // plane ahead of its use: the columns' plane z + 2, the halo's plane z + 1.  The
@@ -512,45 +512,58 @@ __global__ void __launch_bounds__(kMarchTX* kMarchTY) k_sweep_march(Geo g, const
 // (4.6 TB/s of the 36 B a node; 15.8 M warp instructions against 21.4 M), with the
 // IB 49.3 against 51.0; 72x72x384 27.2 against 30.7; 89x89x300 (one scalar node
 // per thread before) 31.7 against 36.5.  (L2 eviction hints on u, b or the new b:
-// 39.8 to 44 us at 96x96x512.)  The batch keeps march_tile: its small members
-// leave most of a 32 x 16 tile idle (12 pipes of 40^2 to 58^2 44.9 ms against 40.1).
-constexpr int kPairTXP = 16, kPairTY = 16;
-constexpr int kPairThreads = kPairTXP * kPairTY / 2;
+// 39.8 to 44 us at 96x96x512.)  The joint march of a batch keeps march_tile: small
+// members leave most of a 32 x 16 tile idle (12 pipes of 40^2 to 58^2 44.9 ms against
+// 40.1).
+//
+// A domain of less than a wave of tiles is bound by the time of one CTA, its chunk's
+// planes one after the other: there a thread takes one row, and the chunk is as short
+// as one wave allows (pair_shape).  Sweep alone, two rows and at least four planes a
+// chunk / now: 64x64x128 7.4 / 6.0 us, 48x48x128 7.6 / 5.0, 40x40x192 7.6 / 5.9,
+// 101x101x20 9.2 / 4.8, 128x128x16 7.7 / 4.0.
+constexpr int kPairTXP = 16, kPairThreads = 128;
+template <int R>
+constexpr int kPairTY = 8 * R;
 // Floats between two rows of a staged half: a warp covers two thread rows, two
 // tile rows apart, whose 16 columns have to lie 16 banks apart (17, unpadded, puts
 // them 2 banks apart).
 constexpr int kPairRow = 24;
 // Floats of one half (even or odd columns) of a field in the staged tile.
-constexpr int kPairHalf = (kPairTY + 2) * kPairRow;
-static_assert(2 * kPairTXP + 2 * kPairTY <= kPairThreads, "one halo item a thread");
+template <int R>
+constexpr int kPairHalf = (kPairTY<R> + 2) * kPairRow;
+// CTAs kept resident per SM (bounds the registers: 162 at two rows, 114 at one).
+template <int R>
+constexpr int kPairMinBlocks = R == 2 ? 3 : 4;
 // [buffer][field][even, odd][row][column]; rows: the tile's and one halo row on
 // each side; even column c is node 2c (one past the last: the halo right of the
 // tile), odd column c is node 2c - 1 (0: the halo left of it)
-using PairTile = float[2][6][2][kPairHalf];
+template <int R>
+using PairTile = float[2][6][2][kPairHalf<R>];
 
 // Halo item hid of a pair tile: the pairs of the row above, of the row below, the
 // nodes of the column left of the tile, of the column right of it (corners are not
 // needed by the 5-point in-plane stencil).  kind: 0 none, 1 pair, 2 left node,
 // 3 right node; at: its offset in a staged half; gp, gq: in-plane indices of its
 // nodes (periodic images).
+template <int TY>
 __device__ __forceinline__ void pair_halo(int hid, int x0, int y0, int nx, int ny, int& kind, int& at, int& gp,
                                           int& gq) {
     kind = 0;
     at = 0;
     gp = gq = 0;
-    if (hid >= 2 * kPairTXP + 2 * kPairTY) return;
+    if (hid >= 2 * kPairTXP + 2 * TY) return;
     if (hid < 2 * kPairTXP) {
         const bool above = hid < kPairTXP;
         const int col = above ? hid : hid - kPairTXP;
         kind = 1;
-        at = (above ? 0 : kPairTY + 1) * kPairRow + col;
-        const int gx = (x0 + 2 * col) % nx, gy = above ? (y0 - 1 + ny) % ny : (y0 + kPairTY) % ny;
+        at = (above ? 0 : TY + 1) * kPairRow + col;
+        const int gx = (x0 + 2 * col) % nx, gy = above ? (y0 - 1 + ny) % ny : (y0 + TY) % ny;
         gp = gy * nx + gx;
         gq = gy * nx + (gx + 1) % nx;
     } else {
         const int j = hid - 2 * kPairTXP;
-        const bool left = j < kPairTY;
-        const int i = left ? j : j - kPairTY;
+        const bool left = j < TY;
+        const int i = left ? j : j - TY;
         kind = left ? 2 : 3;
         at = (1 + i) * kPairRow + (left ? 0 : kPairTXP);
         const int gx = left ? (x0 - 1 + nx) % nx : (x0 + 2 * kPairTXP) % nx;
@@ -586,26 +599,35 @@ __device__ __forceinline__ float2 pair_update(float w0, float w1, float w1k, flo
     return fma2(f2(w0, w0), b, fma2(f2(w1k, w1k), d, mul2(f2(w1, w1), s)));
 }
 
-template <bool XY>
+template <bool XY, int R>
 __device__ __forceinline__ void pair_tile(const Geo& g, const float* __restrict__ bin, float* __restrict__ bout,
                                           const float* __restrict__ u, const SweepCoef<float>& c, int bx, int by,
-                                          int bz, int chunk, PairTile& tile) {
+                                          int bz, int chunk, PairTile<R>& tile) {
     const int nx = g.nx, ny = g.ny, nz = g.nz;
     const int n = (int)g.n, P = nx * ny;
     const bool even = (nx & 1) == 0;  // pairs lie on 8-byte boundaries
-    const int tx = threadIdx.x % kPairTXP, ty = threadIdx.x / kPairTXP;
-    const int x0 = bx * 2 * kPairTXP, y0 = by * kPairTY;
-    const int x = x0 + 2 * tx, y = y0 + 2 * ty;
-    const bool active[2] = {x < nx && y < ny, x < nx && y + 1 < ny};
+    constexpr int TY = kPairTY<R>, half = kPairHalf<R>;
+    static_assert(kPairTXP * TY == R * kPairThreads && 2 * kPairTXP + 2 * TY <= kPairThreads, "one halo item a thread");
+    const int tx = threadIdx.x % kPairTXP, trow = threadIdx.x / kPairTXP;
+    // the thread's first row: a warp's two thread rows lie two tile rows apart
+    const int ty = R == 2 ? 2 * trow : (trow & ~3) + ((trow >> 1) & 1) + 2 * (trow & 1);
+    const int x0 = bx * 2 * kPairTXP, y0 = by * TY;
+    const int x = x0 + 2 * tx, y = y0 + ty;
     // rows and columns past the domain's end stage the periodic images their
     // neighbours need; p: the pairs' first nodes, dq: from there to the second
-    const int p[2] = {(y % ny) * nx + (x % nx), ((y + 1) % ny) * nx + (x % nx)};
+    bool active[R];
+    int p[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        active[r] = x < nx && y + r < ny;
+        p[r] = ((y + r) % ny) * nx + (x % nx);
+    }
     const int dq = x % nx == nx - 1 ? 1 - nx : 1;
     const bool two = x + 1 < nx;  // the second node is in the domain
     const int z0 = bz * chunk;
     const int z1 = min(z0 + chunk, nz);
     int hkind, hat, hp, hq;
-    pair_halo(threadIdx.x, x0, y0, nx, ny, hkind, hat, hp, hq);
+    pair_halo<TY>(threadIdx.x, x0, y0, nx, ny, hkind, hat, hp, hq);
     // nodes k and k + d
     auto load = [&](int k, int d, float2 r[6]) {
         if (even) {
@@ -648,18 +670,18 @@ __device__ __forceinline__ void pair_tile(const Geo& g, const float* __restrict_
             pair_emf(r, be, be, c.sq);
         }
     };
-    float2 prv[2][6], cur[2][6], nxt[2][6], ahd[2][6], halo[6];
+    float2 prv[R][6], cur[R][6], nxt[R][6], ahd[R][6], halo[6];
     {
         const int zm = wrap_dec(z0, nz), zn = wrap_inc(z0, nz);
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
+        for (int r = 0; r < R; ++r) {
             load(zm * P + p[r], dq, prv[r]);
             load(z0 * P + p[r], dq, cur[r]);
             load(zn * P + p[r], dq, nxt[r]);
         }
         load_halo(z0, halo);
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
+        for (int r = 0; r < R; ++r) {
             emf2(prv[r], zm, p[r], dq);
             emf2(cur[r], z0, p[r], dq);
             emf2(nxt[r], zn, p[r], dq);
@@ -667,18 +689,19 @@ __device__ __forceinline__ void pair_tile(const Geo& g, const float* __restrict_
     }
     const float w0 = c.w0, w1 = c.w1, w1k = c.w1 * c.kappa;
     constexpr int rs = kPairRow;
-    const int at = (2 * ty + 1) * rs + tx;  // the pair's place in the halves
+    const int at = (ty + 1) * rs + tx;  // the pair's place in the halves
     for (int z = z0; z < z1; ++z) {
         const int zn = wrap_inc(z, nz);
         const int za = wrap_inc(zn, nz);
         auto& t = tile[z & 1];
-        float* const te = &t[0][0][at];  // fields 2 kPairHalf apart, the odd half kPairHalf on
+        float* const te = &t[0][0][at];  // fields 2 half apart, the odd half half on
 #pragma unroll
         for (int v = 0; v < 6; ++v) {
-            te[2 * v * kPairHalf] = cur[0][v].x;
-            te[2 * v * kPairHalf + kPairHalf + 1] = cur[0][v].y;
-            te[2 * v * kPairHalf + rs] = cur[1][v].x;
-            te[2 * v * kPairHalf + kPairHalf + 1 + rs] = cur[1][v].y;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                te[2 * v * half + r * rs] = cur[r][v].x;
+                te[2 * v * half + half + 1 + r * rs] = cur[r][v].y;
+            }
         }
         if (hkind != 0) {
             emf2(halo, z, hp, hq - hp);  // a single halo node uses .x only
@@ -698,32 +721,32 @@ __device__ __forceinline__ void pair_tile(const Geo& g, const float* __restrict_
         }
         if (z + 1 < z1) {
 #pragma unroll
-            for (int r = 0; r < 2; ++r) load(za * P + p[r], dq, ahd[r]);
+            for (int r = 0; r < R; ++r) load(za * P + p[r], dq, ahd[r]);
             load_halo(zn, halo);
         }
         __syncthreads();
-        // rows above and below the thread's two: b, e1, e3
+        // rows above and below the thread's: b, e1, e3
         float2 up[6], dn[6];
         {
-            const float *tu = te - rs, *td = te + 2 * rs;
+            const float *tu = te - rs, *td = te + R * rs;
 #pragma unroll
             for (int v = 0; v < 6; ++v)
                 if (v != 4) {
-                    up[v] = f2(tu[2 * v * kPairHalf], tu[2 * v * kPairHalf + kPairHalf + 1]);
-                    dn[v] = f2(td[2 * v * kPairHalf], td[2 * v * kPairHalf + kPairHalf + 1]);
+                    up[v] = f2(tu[2 * v * half], tu[2 * v * half + half + 1]);
+                    dn[v] = f2(td[2 * v * half], td[2 * v * half + half + 1]);
                 }
         }
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
+        for (int r = 0; r < R; ++r) {
             const float2* a_ = r == 0 ? up : cur[0];  // the row above
-            const float2* b_ = r == 0 ? cur[1] : dn;  // the row below
+            const float2* b_ = r == R - 1 ? dn : cur[R - 1];  // the row below
             const float2* o = cur[r];
             const float* tr = te + r * rs;
             float lf[5], rt[5];  // x neighbours: b, e1, e2
 #pragma unroll
             for (int v = 0; v < 5; ++v) {
-                lf[v] = tr[2 * v * kPairHalf + kPairHalf];
-                rt[v] = tr[2 * v * kPairHalf + 1];
+                lf[v] = tr[2 * v * half + half];
+                rt[v] = tr[2 * v * half + 1];
             }
             const float2 d[3] = {
                 add2(sub2(b_[3], a_[3]), sub2(nxt[r][4], prv[r][4])),
@@ -747,7 +770,7 @@ __device__ __forceinline__ void pair_tile(const Geo& g, const float* __restrict_
             }
         }
 #pragma unroll
-        for (int r = 0; r < 2; ++r)
+        for (int r = 0; r < R; ++r)
 #pragma unroll
             for (int v = 0; v < 6; ++v) {
                 prv[r][v] = cur[r][v];
@@ -755,7 +778,7 @@ __device__ __forceinline__ void pair_tile(const Geo& g, const float* __restrict_
             }
         if (z + 1 < z1) {
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
+            for (int r = 0; r < R; ++r) {
                 emf2(ahd[r], za, p[r], dq);
 #pragma unroll
                 for (int v = 0; v < 6; ++v) nxt[r][v] = ahd[r][v];
@@ -764,17 +787,17 @@ __device__ __forceinline__ void pair_tile(const Geo& g, const float* __restrict_
     }
 }
 
-template <typename F, bool XY>
-__global__ void __launch_bounds__(kPairThreads, 3) k_sweep_march_pair(Geo g, const F* __restrict__ bin,
-                                                                      F* __restrict__ bout, const F* __restrict__ u,
-                                                                      SweepCoef<F> c, int chunk) {
+template <typename F, bool XY, int R>
+__global__ void __launch_bounds__(kPairThreads, kPairMinBlocks<R>)
+    k_sweep_march_pair(Geo g, const F* __restrict__ bin, F* __restrict__ bout, const F* __restrict__ u,
+                       SweepCoef<F> c, int chunk) {
     static_assert(sizeof(F) == 4, "the pair sweep is the FP32 path");
-    __shared__ __align__(16) PairTile tile;
+    __shared__ __align__(16) PairTile<R> tile;
     // the IB pass after this sweep may be scheduled as this grid's CTAs exit;
     // b comes from the kernel before this one
     pdl_trigger();
     pdl_wait();
-    pair_tile<XY>(g, bin, bout, u, c, blockIdx.x, blockIdx.y, blockIdx.z, chunk, tile);
+    pair_tile<XY, R>(g, bin, bout, u, c, blockIdx.x, blockIdx.y, blockIdx.z, chunk, tile);
 }
 
 // Two-phase IB corrector over the whole domain (Sec. V.C-V.F): first one

@@ -143,15 +143,12 @@ struct Launch {
                 T* bout = (T*)s.b[1 - s.bcur];
                 const T* u = (const T*)s.u[s.fcur];
                 if (pair_march(s)) {
+                    const auto kern = pair_kernel(s.bext_xy != nullptr, s.march_rows);
+                    const int ty = 8 * s.march_rows;
                     const dim3 pgrid((unsigned)((s.nx + 2 * kPairTXP - 1) / (2 * kPairTXP)),
-                                     (unsigned)((s.ny + kPairTY - 1) / kPairTY),
-                                     (unsigned)((s.nz + chunk - 1) / chunk));
-                    if (s.bext_xy)
-                        launch_pdl(k_sweep_march_pair<float, true>, pgrid, dim3(kPairThreads), 0, st, geo(s),
-                                   (const float*)bin, (float*)bout, (const float*)u, fcoef(c), chunk);
-                    else
-                        launch_pdl(k_sweep_march_pair<float, false>, pgrid, dim3(kPairThreads), 0, st, geo(s),
-                                   (const float*)bin, (float*)bout, (const float*)u, fcoef(c), chunk);
+                                     (unsigned)((s.ny + ty - 1) / ty), (unsigned)((s.nz + chunk - 1) / chunk));
+                    launch_pdl(kern, pgrid, dim3(kPairThreads), 0, st, geo(s), (const float*)bin, (float*)bout,
+                               (const float*)u, fcoef(c), chunk);
                 } else if (s.dim == 3) {
                     if (s.bext_xy)
                         k_sweep_march<T, true><<<mgrid, kMarchTX * kMarchTY, 0, st>>>(geo(s), bin, bout, u, c, chunk);
@@ -532,11 +529,15 @@ struct Launch {
             *out = {QSLBM_KERNEL_NODES, (s.nx * s.ny + kNodeThreads - 1) / kNodeThreads, kNodeThreads, 0, 1};
         else {
             const bool pair = s.march_rows > 0;
-            const int tx = pair ? 2 * kPairTXP : kMarchTX, ty = pair ? kPairTY : kMarchTY;
+            const int tx = pair ? 2 * kPairTXP : kMarchTX, ty = pair ? 8 * s.march_rows : kMarchTY;
             *out = {pair ? QSLBM_KERNEL_MARCH_PAIR : QSLBM_KERNEL_MARCH,
                     ((s.nx + tx - 1) / tx) * ((s.ny + ty - 1) / ty) * ((s.nz + s.march_chunk - 1) / s.march_chunk),
                     pair ? kPairThreads : kMarchTX * kMarchTY, s.march_rows, s.march_chunk};
         }
+    }
+    static auto pair_kernel(bool xy, int rows) {
+        return rows == 1 ? (xy ? k_sweep_march_pair<float, true, 1> : k_sweep_march_pair<float, false, 1>)
+                         : (xy ? k_sweep_march_pair<float, true, 2> : k_sweep_march_pair<float, false, 2>);
     }
     static SweepCoef<float> fcoef(const SweepCoef<T>& c) {
         if constexpr (sizeof(T) == 4)
@@ -545,38 +546,66 @@ struct Launch {
             return SweepCoef<float>{};  // never launched: the pair kernel is FP32 only
     }
 
-    // z planes per CTA of the marching sweep such that the grid fills one wave
-    static cudaError_t plan_march(State& s) {
+    // z planes per CTA such that a grid of tiles of tx x ty columns fills one wave of
+    // the kernel's resident CTAs (`share`: of which so many such grids run at a time),
+    // at least `least`.
+    static cudaError_t wave_chunk(const State& s, const void* kern, int threads, int tx, int ty, int least, int share,
+                                  int& chunk) {
         int dev = 0, sms = 0, per_sm = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const bool pair = pair_march(s);
-        if (e == cudaSuccess) {
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, 0);
+        const long long tiles = (long long)((s.nx + tx - 1) / tx) * ((s.ny + ty - 1) / ty);
+        const long long slots = (long long)std::max(1, per_sm) * std::max(1, sms) / share;
+        const long long per_column = std::max<long long>(1, slots / tiles);
+        chunk = (int)std::min<long long>(std::max<long long>((s.nz + per_column - 1) / per_column, least), s.nz);
+        return e;
+    }
+
+    // The pair sweep's rows per thread and planes per CTA, on a domain that shares the
+    // device with share - 1 others: one wave either way.  Two rows (chunk c2) where a
+    // CTA's chunk is of four planes or more; below, the time is that of one CTA's chain
+    // of planes, and a plane costs one row a thread (chunk c1) about 0.7 of what it costs
+    // two.  Sweep alone, us: 64x64x128 c2 = 3 6.2, c1 = 4 6.0; 48x48x128 c2 = 2 5.0, c1 =
+    // 3 5.1; 128x128x16 c2 = 2 4.9, c1 = 2 4.0; 40x40x300 c2 = 4 7.5, c1 = 5 8.1 (chunks of
+    // at least four planes: 7.4, 7.6, 7.7, 7.5).  A grid that would need more than four
+    // planes only because of the others keeps four.
+    static cudaError_t pair_shape(const State& s, int share, int* rows, int* chunk) {
+        const bool xy = s.bext_xy != nullptr;
+        const void *k1 = (const void*)pair_kernel(xy, 1), *k2 = (const void*)pair_kernel(xy, 2);
+        int c1 = 1, c2 = 1, alone = 1;
+        cudaError_t e = wave_chunk(s, k2, kPairThreads, 2 * kPairTXP, kPairTY<2>, 1, 1, alone);
+        if (e == cudaSuccess) e = wave_chunk(s, k2, kPairThreads, 2 * kPairTXP, kPairTY<2>, 1, share, c2);
+        if (e == cudaSuccess) e = wave_chunk(s, k1, kPairThreads, 2 * kPairTXP, kPairTY<1>, 1, share, c1);
+        c2 = std::min(c2, std::max(alone, 4));
+        *rows = c2 < 4 && 10 * c1 <= 14 * c2 ? 1 : 2;
+        *chunk = *rows == 1 ? c1 : c2;
+        return e;
+    }
+
+    // The marching sweep's planes per CTA and, for pairs, rows per thread.
+    static cudaError_t plan_march(State& s) {
+        cudaError_t e;
+        if (pair_march(s)) {
+            e = pair_shape(s, 1, &s.march_rows, &s.march_chunk);
+        } else {
             const void* kern = (const void*)k_sweep_march<T, true>;
-            if constexpr (sizeof(T) == 4) {
-                if (pair)
-                    kern = s.bext_xy ? (const void*)k_sweep_march_pair<T, true> : (const void*)k_sweep_march_pair<T, false>;
-            } else if (!s.bext_xy) {
-                kern = (const void*)k_sweep_march<T, false>;
-            }
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, pair ? kPairThreads : kMarchTX * kMarchTY, 0);
+            if constexpr (sizeof(T) == 8)
+                if (!s.bext_xy) kern = (const void*)k_sweep_march<T, false>;
+            // (at least four planes, to keep the z halo's share small)
+            e = wave_chunk(s, kern, kMarchTX * kMarchTY, kMarchTX, kMarchTY, 4, 1, s.march_chunk);
+            s.march_rows = 0;
         }
         if (e != cudaSuccess) return e;
-        const int tx = pair ? 2 * kPairTXP : kMarchTX, ty = pair ? kPairTY : kMarchTY;
-        const long long tiles = (long long)((s.nx + tx - 1) / tx) * ((s.ny + ty - 1) / ty);
-        const long long slots = (long long)std::max(1, per_sm) * std::max(1, sms);
-        const long long per_column = std::max<long long>(1, slots / std::max<long long>(1, tiles));
-        long long chunk = (s.nz + per_column - 1) / per_column;
-        chunk = std::max<long long>(chunk, 4);  // keep the z halo overhead small
-        s.march_chunk = (int)std::min<long long>(chunk, s.nz);
-        s.march_rows = pair ? 2 : 0;
         // the staged IB corrector, when the plane's shell fits shared memory
         // and the shell nodes' marker lists are padded
         s.ib_staged_smem = 0;
         if (s.ib.nm > 0 && s.ib.pad_k > 0) {
             const size_t smem = ib_staged_smem_bytes<T>(s.ib.max_ring, s.ib.max_shell);
-            int max_optin = 0;
-            e = cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+            int dev = 0, sms = 0, max_optin = 0;
+            e = cudaGetDevice(&dev);
+            if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            if (e == cudaSuccess) e = cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
             if (e != cudaSuccess) return e;
             if (smem <= (size_t)max_optin) {
                 s.ib_staged_u = ib_staged_unroll(s.ib.max_shell, s.nz, sms);
@@ -846,7 +875,7 @@ struct Launch {
 
     static const Ops& table() {
         static const Ops o = {&init,     &sweeps,        &force_flow, &observe,     &observe_fields,
-                              &to_f64,   &from_f64,      &plan_resident, &plan_march, &sweep_plan,
+                              &to_f64,   &from_f64,      &plan_resident, &plan_march, &pair_shape, &sweep_plan,
                               &plan_fused, &tune_fused};
         return o;
     }
