@@ -218,7 +218,8 @@ int qslbm_get_units(const qslbm_handle* h, qslbm_units* out);
  *   threads  threads per CTA
  *   rows     SLAB, MARCH_PAIR: rows per thread; CLUSTER64: rows per CTA;
  *            FUSED: rows per band; else 0
- *   planes   z planes per CTA, at most */
+ *   planes   z planes per CTA, at most
+ *   ib_early MARCH_PAIR, MARCH: 1 when the IB pass's CTAs start as the sweep's end */
 #define QSLBM_KERNEL_PLANES 1     /* k_sweep_ib: one sweep and its IB per launch, a plane per CTA */
 #define QSLBM_KERNEL_RESIDENT 2   /* k_sweeps_resident: all sweeps, a plane per CTA */
 #define QSLBM_KERNEL_SLAB 3       /* k_sweeps_slab: all sweeps (FP32), planes per CTA as needed */
@@ -229,7 +230,7 @@ int qslbm_get_units(const qslbm_handle* h, qslbm_units* out);
 #define QSLBM_KERNEL_MARCH 8      /* k_sweep_march, then the IB */
 #define QSLBM_KERNEL_NODES 9      /* k_sweep_nodes (2-D), then the IB */
 typedef struct qslbm_sweep_plan_t {
-    int32_t kernel, ctas, threads, rows, planes;
+    int32_t kernel, ctas, threads, rows, planes, ib_early;
 } qslbm_sweep_plan_t;
 /* Errors: QSLBM_EINVAL (NULL argument). */
 int qslbm_sweep_plan(const qslbm_handle* h, qslbm_sweep_plan_t* out);

@@ -54,7 +54,7 @@ class qslbm_units(C.Structure):
 
 
 class qslbm_sweep_plan_t(C.Structure):
-    _fields_ = [(k, C.c_int32) for k in ("kernel", "ctas", "threads", "rows", "planes")]
+    _fields_ = [(k, C.c_int32) for k in ("kernel", "ctas", "threads", "rows", "planes", "ib_early")]
 
 
 SWEEP_PLAN_KERNEL = {1: "k_sweep_ib", 2: "k_sweeps_resident", 3: "k_sweeps_slab", 4: "k_sweeps_resident64",

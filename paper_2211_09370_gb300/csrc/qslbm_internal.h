@@ -116,6 +116,7 @@ struct State {
     int march_chunk = 16;       // z planes per CTA of the marching sweep (one wave)
     int march_rows = 0;         // rows per thread of the FP32 pair sweep (0: one node per thread)
     size_t ib_staged_smem = 0;  // shared memory of k_ib_staged, 0 when it does not fit
+    bool ib_early = false;      // k_ib_staged on b may start as the sweep before it ends
     int ib_staged_u = 1;        // its shell nodes per thread per batch of loads (1, 2, 4 or 5)
     bool resident_uhalo = false;
     size_t resident_smem = 0;

@@ -45,9 +45,9 @@ struct Launch {
 
     // A launch that may begin while the previous kernel in the stream finishes
     // (programmatic dependent launch; the kernel calls pdl_wait before it
-    // touches that kernel's results).
+    // touches that kernel's results), or, without `early`, an ordinary one.
     template <typename... KArgs, typename... Args>
-    static void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+    static void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool early,
                            Args... args) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = grid;
@@ -56,7 +56,7 @@ struct Launch {
         cfg.stream = st;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        attr[0].val.programmaticStreamSerializationAllowed = early;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         cudaLaunchKernelEx(&cfg, kernel, args...);  // errors surface at the next synchronising call
@@ -79,16 +79,17 @@ struct Launch {
                                                        s.units.U0, s.axis);
     }
 
-    // The staged IB corrector on every plane of f.
-    static void launch_ib_staged(const State& s, T* f, const IBView<T>& v, cudaStream_t st) {
+    // The staged IB corrector on every plane of f; early: scheduled as the CTAs of the
+    // kernel before it exit.
+    static void launch_ib_staged(const State& s, T* f, const IBView<T>& v, bool early, cudaStream_t st) {
         const int R = s.ib.max_ring, S = s.ib.max_shell;
         const size_t sm = s.ib_staged_smem;
         const dim3 ig((unsigned)s.nz), ib(kNodeThreads);
         switch (s.ib_staged_u) {
-            case 1: launch_pdl(k_ib_staged<T, 1>, ig, ib, sm, st, geo(s), f, v, R, S); break;
-            case 2: launch_pdl(k_ib_staged<T, 2>, ig, ib, sm, st, geo(s), f, v, R, S); break;
-            case 4: launch_pdl(k_ib_staged<T, 4>, ig, ib, sm, st, geo(s), f, v, R, S); break;
-            default: launch_pdl(k_ib_staged<T, 5>, ig, ib, sm, st, geo(s), f, v, R, S); break;
+            case 1: launch_pdl(k_ib_staged<T, 1>, ig, ib, sm, st, early, geo(s), f, v, R, S); break;
+            case 2: launch_pdl(k_ib_staged<T, 2>, ig, ib, sm, st, early, geo(s), f, v, R, S); break;
+            case 4: launch_pdl(k_ib_staged<T, 4>, ig, ib, sm, st, early, geo(s), f, v, R, S); break;
+            default: launch_pdl(k_ib_staged<T, 5>, ig, ib, sm, st, early, geo(s), f, v, R, S); break;
         }
     }
 
@@ -147,7 +148,7 @@ struct Launch {
                     const int ty = 8 * s.march_rows;
                     const dim3 pgrid((unsigned)((s.nx + 2 * kPairTXP - 1) / (2 * kPairTXP)),
                                      (unsigned)((s.ny + ty - 1) / ty), (unsigned)((s.nz + chunk - 1) / chunk));
-                    launch_pdl(kern, pgrid, dim3(kPairThreads), 0, st, geo(s), (const float*)bin, (float*)bout,
+                    launch_pdl(kern, pgrid, dim3(kPairThreads), 0, st, true, geo(s), (const float*)bin, (float*)bout,
                                (const float*)u, fcoef(c), chunk);
                 } else if (s.dim == 3) {
                     if (s.bext_xy)
@@ -158,7 +159,7 @@ struct Launch {
                     k_sweep_nodes<T, 2><<<grid, kNodeThreads, 0, st>>>(geo(s), bin, bout, u, c);
                 }
                 if (s.ib.nm > 0 && s.ib_staged_smem > 0) {
-                    launch_ib_staged(s, bout, v, st);
+                    launch_ib_staged(s, bout, v, s.ib_early, st);
                 } else if (s.ib.nm > 0) {
                     k_ib_markers<T><<<(s.ib.nm + kNodeThreads - 1) / kNodeThreads, kNodeThreads, 0, st>>>(geo(s), bout, v);
                     k_ib_shell<T><<<(s.ib.ns + kNodeThreads - 1) / kNodeThreads, kNodeThreads, 0, st>>>(geo(s), bout, v);
@@ -242,7 +243,7 @@ struct Launch {
             const dim3 grid((unsigned)s.fu_bands, (unsigned)s.fu_chunks);
             const FusedGeo g{s.nx, s.ny, s.nz, s.fu_TY, s.fu_chunk, (int)s.n, s.fu_slots};
             const int bc = s.bcur, fc = s.fcur;
-            launch_pdl(fused_kernel(s), grid, dim3(s.fu_threads), s.fu_smem, st, s.fu_map_b3[bc], s.fu_map_bt[bc],
+            launch_pdl(fused_kernel(s), grid, dim3(s.fu_threads), s.fu_smem, st, true, s.fu_map_b3[bc], s.fu_map_bt[bc],
                        s.fu_map_u3[fc], s.fu_map_ut[fc], (float*)s.b[1 - bc], c, fused_ib(s), g, s.fu_err);
         } else {
             s.launch_error = true;  // never planned: the fused sweep is the FP32 path
@@ -532,7 +533,7 @@ struct Launch {
             const int tx = pair ? 2 * kPairTXP : kMarchTX, ty = pair ? 8 * s.march_rows : kMarchTY;
             *out = {pair ? QSLBM_KERNEL_MARCH_PAIR : QSLBM_KERNEL_MARCH,
                     ((s.nx + tx - 1) / tx) * ((s.ny + ty - 1) / ty) * ((s.nz + s.march_chunk - 1) / s.march_chunk),
-                    pair ? kPairThreads : kMarchTX * kMarchTY, s.march_rows, s.march_chunk};
+                    pair ? kPairThreads : kMarchTX * kMarchTY, s.march_rows, s.march_chunk, s.ib_early};
         }
     }
     static auto pair_kernel(bool xy, int rows) {
@@ -617,6 +618,12 @@ struct Launch {
                 e = allow_smem((const void*)kern, smem);
                 if (e != cudaSuccess) return e;
                 s.ib_staged_smem = smem;
+                // Early CTAs gather on the SMs whose sweep CTAs end first, two and more to
+                // an SM: where the planes have an SM each, spreading them is worth more
+                // than the earlier start (us a sweep, early / not: 99x99x64 16.6 / 14.3,
+                // 96x96x40 12.1 / 9.3, 128x128x60 23.6 / 17.3, 64x64x128 10.6 / 9.6; with
+                // more planes than SMs 40x40x192 8.6 / 9.3, 96x96x512 48.8 / 51.7).
+                s.ib_early = s.nz > sms;
             }
         }
         return cudaSuccess;
@@ -819,7 +826,7 @@ struct Launch {
             }
         }
         if (s.ib.nm > 0 && s.ib_staged_smem > 0)
-            launch_ib_staged(s, uo, v, st);
+            launch_ib_staged(s, uo, v, true, st);
         else if (s.ib.nm > 0)
             k_ib_planes<T><<<s.nz, kNodeThreads, ib_smem(s), st>>>(geo(s), uo, v);
         s.fcur ^= 1;

@@ -41,6 +41,6 @@ def test_plan_names_every_kernel_of_the_header():
         src = f.read()
     names = {int(v): c for v, c in re.findall(r"#define QSLBM_KERNEL_\w+ (\d+)\s*/\* (\w+)", src)}
     assert names == _lib.SWEEP_PLAN_KERNEL
-    assert C.sizeof(_lib.qslbm_sweep_plan_t) == 20
+    assert C.sizeof(_lib.qslbm_sweep_plan_t) == 24
     L = _lib.load()
     assert L.qslbm_sweep_plan(None, None) == _lib.EINVAL

@@ -57,6 +57,16 @@ def test_small_domains_are_cut_into_short_chunks(shape):
     assert plan["planes"] == 1 or plan["ctas"] >= 2 * sms, plan
 
 
+@pytest.mark.parametrize("shape", [(33, 35, 40), (99, 99, 64), (24, 24, 152), (24, 24, 153), (41, 41, 300)], ids=str)
+def test_ib_pass_waits_where_the_planes_have_an_sm_each(shape):
+    import torch
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    nx, ny, nz = shape
+    with Solver(W.small_pipe(nx=nx, ny=ny, nz=nz, diameter=float(nx - 8), sweep_kernel="split")) as s:
+        assert s.plan()["ib_early"] == (nz > sms)
+
+
 def test_large_domains_keep_two_rows():
     with Solver(W.pipe_ramp_96x96x512(sweep_kernel="split")) as s:
         plan = s.plan()
