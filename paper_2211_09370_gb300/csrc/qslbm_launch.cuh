@@ -359,6 +359,46 @@ struct Launch {
         if (e != cudaSuccess) s.launch_error = true;
     }
 
+    // Estimated us per sweep, where k_sweeps_resident does not apply: of the slab kernel
+    // with K rows a thread and `columns` threads at work on slabs of G planes, its start
+    // (tables, S) included, and of the split sweep and its IB pass.  A slab's time is that
+    // of one CTA, however many there are; the split sweep's grows with the planes of its
+    // chunk (pair_shape), so that a device half full of slabs can lose to it.  Fitted to
+    // 740 domains with and without walls, ramps and in-plane fields.  Measured, slab /
+    // split: 57x57 (five rows) x153 16.4 / 11.6, x245 16.6 / 15.1, x304 16.6 / 17.0; 54x54
+    // (four) x153 13.5 / 9.8, x245 13.5 / 13.1, x304 13.6 / 15.1; without walls 53x53 (four)
+    // x200 11.6 / 8.8, 37x37 (two) x153 6.3 / 5.4; 20x300x40 in an in-plane field 13.2 /
+    // 8.4.  A step of few sweeps does not earn the start back: 40x40x192 (three) at 5
+    // sweeps 89 us a step against 67, at 40 358 against 368.
+    static double slab_us(const State& s, int K, int columns, int G) {
+        const int XP = slab_pairs(s.nx);
+        double t;
+        if (K == 1)
+            t = 1.0 + 0.0022 * columns;
+        else if (K == 2)  // (rows of an odd number of pairs, unpadded, conflict in their banks)
+            t = XP % 2 && slab_row_stride(s.nx, s.ny, G, K) == XP ? 2.6 + 0.0052 * columns : 0.0066 * columns;
+        else if (K == 3)
+            t = G > 1 ? 1.65 + 0.0068 * columns : 3.5 + 0.0033 * columns;
+        else if (K == 4)  // (wide planes, and slabs of several low ones, have fewer conflicts)
+            t = (XP >= 32 ? 0.0125 : G > 2 ? 0.0132 : 0.0155) * columns;
+        else
+            t = 6.3 + 0.01 * columns;
+        const double ib[] = {0.8, 1.5, G > 1 ? 2.0 : 1.0, 1.9, 3.0};
+        if (s.ib.nm > 0) t += ib[K - 1];
+        const double start = 9.0 + 0.0037 * G * s.nx * s.ny + (s.bext_xy ? 3.5 : 0.0);
+        return t + start / std::max(1, s.units.n_mag);
+    }
+    static cudaError_t split_us(const State& s, double* us) {
+        int rows = 2, chunk = 1;
+        const cudaError_t e = pair_shape(s, 1, &rows, &chunk);
+        double t = rows == 1 ? 1.7 + 1.03 * chunk : 1.55 + 1.42 * chunk;
+        if (s.nx % 2) t += rows == 1 ? 1.0 : 1.0 + 0.1 * chunk;
+        if (s.bext_xy) t *= s.nx % 2 ? 1.2 : 1.3;
+        if (s.ib.nm > 0) t += 2.2 + 0.004 * s.ib.max_shell;
+        *us = t;
+        return e;
+    }
+
     // The slab kernel for this domain: the fewest planes per CTA at which every
     // CTA is co-resident.
     static cudaError_t plan_slab(State& s, int optin, int sms) {
@@ -374,12 +414,18 @@ struct Launch {
         // at one row 24x24: 2.0 against 3.6, 36x36: 3.3 against 4.0), whose pairs an
         // odd width does without (47x46: 5.3 against 6.8); even-width slabs of
         // several planes at five rows stay with the marching sweep (60x60x304: 17.6
-        // against 16.4; at three rows 40x40x192: 7.6 against 10.7, at one row
-        // 24x24x300: 2.8 against 8.8).
+        // against 16.4).
         if (s.nx % 2 == 0 && ((G == 1 && K > 1 && s.resident) || (G > 1 && K == kSlabMaxK))) return cudaSuccess;
         // its start (tables, S) takes about 5 us longer than k_sweeps_resident's: a
         // step of few sweeps does not earn that back
         if (s.resident && s.units.n_mag < 24) return cudaSuccess;
+        if (!s.resident) {
+            double split = 0.0;
+            const cudaError_t e = split_us(s, &split);
+            if (e != cudaSuccess) return e;
+            // (the estimates are within some 5 %)
+            if (slab_us(s, K, G * slab_pairs(s.nx) * ((s.ny + K - 1) / K), G) > 1.05 * split) return cudaSuccess;
+        }
         const int R = s.ib.max_ring, S = s.ib.max_shell;
         int more = 0;
         for (int i = 0; i < S; ++i) more += std::max(0, s.hib.csr_off[i + 1] - s.hib.csr_off[i] - 4);

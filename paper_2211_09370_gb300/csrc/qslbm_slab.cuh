@@ -40,11 +40,10 @@
 // has received the neighbour's data of the sweep between, which the neighbour
 // sent after the barrier that ends its reads.
 //
-// Measured, us per sweep with the IB, this kernel against the route before it:
-// 24x24x96 2.0 / 3.6 (one plane per CTA, k_sweeps_resident), 24x24x300 2.8 / 8.8,
-// 40x40x192 7.6 / 10.7, 57x57x245 16.4 / 15.9, 59x59x290 16.7 / 19.3, 61x61x150 9.4 /
-// 12.3 (marching pair sweep and IB launches),
-// 64x64x128 with an in-plane field 7.1 / 13.3.
+// Measured, us per sweep with the IB, this kernel against the other route there:
+// 24x24x96 2.0 / 3.6 (one plane per CTA, k_sweeps_resident); against the marching pair
+// sweep and its IB launches 24x24x300 2.9 / 6.5, 40x40x192 7.6 / 9.3, 57x57x304 16.5 /
+// 17.8, 61x61x120 9.2 / 11.0, 64x64x128 with an in-plane field 7.1 / 12.7.
 #pragma once
 
 #include "qslbm_kernels.cuh"
