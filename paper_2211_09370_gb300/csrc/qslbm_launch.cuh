@@ -284,42 +284,48 @@ struct Launch {
         }
     }
 
-    // Times one sweep of the fused kernel and one of the split path (each
-    // reads b[bcur] and writes b[1 - bcur], which holds no state) on this
-    // handle's own fields: two sweeps to warm up, then four, CUDA events on
-    // the handle's stream.  Leaves the fused kernel in use when it is the
-    // faster one.
-    // Times both routes (two interleaved rounds of 8 sweeps each after a
-    // warm-up, the faster round kept) and takes the fused kernel only when it
-    // is at least 2 % faster: the split path is the simpler one and wins
-    // ties, so that the choice does not flip on timing noise.  Every timed
-    // sweep reads b[bcur] and writes the other buffer, so the state is left
-    // as it was.
+    // Times the fused kernel and the split path on this handle's own fields and takes
+    // the fused one only when it is at least 2 % faster: the split path is the simpler
+    // one and wins ties, so that the choice does not flip on timing noise.  Both are
+    // timed from a graph, as steps run them: on a stream the split path's second launch
+    // per sweep costs more than in a graph, and 24x24x96 in an in-plane field went to the
+    // fused kernel (7.4 us a sweep) for a split path of 5.5.  Two interleaved rounds of
+    // 8 sweeps each after a warm-up, the faster round kept.  Every timed sweep reads
+    // b[bcur] and writes the other buffer, so the state is left as it was.
     static cudaError_t tune_fused(State& s, double* us_fused, double* us_split) {
+        constexpr int kSweeps = 8;
         cudaEvent_t e0 = nullptr, e1 = nullptr;
+        cudaGraphExec_t run[2] = {nullptr, nullptr};
         cudaError_t e = cudaEventCreate(&e0);
         if (e == cudaSuccess) e = cudaEventCreate(&e1);
         double us[2] = {1e300, 1e300};
-        for (int round = 0; round < 2; ++round) {
+        for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
+            s.fused = k == 0;
+            s.p.sweep_kernel = k == 0 ? QSLBM_SWEEP_FUSED : QSLBM_SWEEP_SPLIT;
+            cudaGraph_t g = nullptr;
+            e = cudaStreamBeginCapture(s.stream, cudaStreamCaptureModeThreadLocal);
+            if (e != cudaSuccess) break;
+            for (int r = 0; r < kSweeps; ++r) {
+                sweeps(s, 1, s.stream);
+                s.bcur ^= 1;  // undo the sweep's swap: the next reads the same b
+            }
+            e = cudaStreamEndCapture(s.stream, &g);
+            if (e == cudaSuccess) e = cudaGraphInstantiate(&run[k], g, 0);
+            if (g) cudaGraphDestroy(g);
+        }
+        for (int round = 0; round < 2; ++round)
             for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
-                s.fused = k == 0;
-                s.p.sweep_kernel = k == 0 ? QSLBM_SWEEP_FUSED : QSLBM_SWEEP_SPLIT;
-                for (int r = 0; r < 2; ++r) {
-                    sweeps(s, 1, s.stream);
-                    s.bcur ^= 1;  // undo the sweep's swap: the next reads the same b
-                }
-                e = cudaEventRecord(e0, s.stream);
-                for (int r = 0; r < 8 && e == cudaSuccess; ++r) {
-                    sweeps(s, 1, s.stream);
-                    s.bcur ^= 1;
-                }
+                e = cudaGraphLaunch(run[k], s.stream);
+                if (e == cudaSuccess) e = cudaEventRecord(e0, s.stream);
+                if (e == cudaSuccess) e = cudaGraphLaunch(run[k], s.stream);
                 if (e == cudaSuccess) e = cudaEventRecord(e1, s.stream);
                 if (e == cudaSuccess) e = cudaEventSynchronize(e1);
                 float ms = 0.f;
                 if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-                us[k] = std::min(us[k], 1e3 * ms / 8);
+                us[k] = std::min(us[k], 1e3 * ms / kSweeps);
             }
-        }
+        for (cudaGraphExec_t x : run)
+            if (x) cudaGraphExecDestroy(x);
         if (e0) cudaEventDestroy(e0);
         if (e1) cudaEventDestroy(e1);
         if (e == cudaSuccess) e = cudaGetLastError();
