@@ -479,7 +479,8 @@ constexpr int kChainStreams = 16;
 constexpr long long kChainInFlight = 1200000;
 
 bool chain_member(const State& s) {
-    return s.esz == 4 && s.dim == 3 && (s.ib.nm == 0 || s.ib_staged_smem > 0);
+    return s.esz == 4 && s.dim == 3 && (s.ib.nm == 0 || s.ib_staged_smem > 0) &&
+           s.ny <= 65535LL * qslbm::kPairTY<2>;  // (a grid's tiles of rows; the joint march has one dimension)
 }
 
 void launch_chain(qslbm_batch& B, int k, cudaStream_t st) {

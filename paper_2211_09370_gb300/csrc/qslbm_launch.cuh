@@ -631,7 +631,8 @@ struct Launch {
         if (e == cudaSuccess) e = wave_chunk(s, k2, kPairThreads, 2 * kPairTXP, kPairTY<2>, 1, share, c2);
         if (e == cudaSuccess) e = wave_chunk(s, k1, kPairThreads, 2 * kPairTXP, kPairTY<1>, 1, share, c1);
         c2 = std::min(c2, std::max(alone, 4));
-        *rows = c2 < 4 && 10 * c1 <= 14 * c2 ? 1 : 2;
+        // (a grid has at most 65535 tiles of rows)
+        *rows = c2 < 4 && 10 * c1 <= 14 * c2 && s.ny <= 65535LL * kPairTY<1> ? 1 : 2;
         *chunk = *rows == 1 ? c1 : c2;
         return e;
     }
