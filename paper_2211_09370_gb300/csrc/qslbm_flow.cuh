@@ -259,7 +259,10 @@ __global__ void __launch_bounds__(kFlowNodeThreads) k_flow_nodes(Geo g, const T*
 // 126 loads through L1, and a third of its arithmetic.  Force, flow and the IB on u
 // of a step, with one CTA per plane gathering from L1 / now: 96x96x512 289 / 131 us
 // (the fields alone are 320 MB, 47 us at the measured copy rate), 40x40x192 51 / 22,
-// 64x64x128 42 / 26, in FP64 about 760 / 200.
+// 64x64x128 42 / 26, in FP64 about 760 / 200.  On small domains, where a step of few
+// sweeps is a handful of launches, force, flow and the IB on u each start as the kernel
+// before them ends (early): 16^3 at one sweep 18.9 us a step without, 16.9 with, 24x24x96
+// at four 32.8 and 31.2.
 constexpr int kFlowTX = 32;
 template <typename T>
 constexpr int kFlowTY = sizeof(T) == 4 ? 8 : 4;  // (the staged planes fit static shared memory)
@@ -301,7 +304,9 @@ __device__ __forceinline__ void flow_halo(int h, int x0, int y0, int nx, int ny,
 template <typename T, int Q>
 __global__ void __launch_bounds__(kFlowThreads<T>) k_force_march(Geo g, const T* __restrict__ b, T* __restrict__ F,
                                                                  ForceCoef<T> c, const long long* __restrict__ tstep,
-                                                                 int chunk) {
+                                                                 int chunk, bool early) {
+    if (early) pdl_trigger();
+    pdl_wait();
     constexpr int TY = kFlowTY<T>, W = kFlowTX + 2, CELLS = W * (TY + 2), HALO = 2 * W + 2 * TY;
     __shared__ T sm[2][3][CELLS];
     static_assert(HALO <= kFlowThreads<T>, "one halo cell a thread");
@@ -363,7 +368,9 @@ template <typename T, int Q>
 __global__ void __launch_bounds__(kFlowThreads<T>) k_flow_march(Geo g, const T* __restrict__ drho,
                                                                 const T* __restrict__ u, const T* __restrict__ F,
                                                                 T* __restrict__ drho_out, T* uout, FlowCoef<T> fc,
-                                                                long long* tstep, int chunk) {
+                                                                long long* tstep, int chunk, bool early) {
+    if (early) pdl_trigger();
+    pdl_wait();
     constexpr int TY = kFlowTY<T>, W = kFlowTX + 2, CELLS = W * (TY + 2), HALO = 2 * W + 2 * TY;
     __shared__ T sm[2][9][CELLS];
     const int nx = g.nx, ny = g.ny, nz = g.nz, P = nx * ny;

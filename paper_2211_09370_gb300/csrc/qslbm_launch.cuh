@@ -56,9 +56,9 @@ struct Launch {
         cfg.stream = st;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = early;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = early ? 1 : 0;
         cudaLaunchKernelEx(&cfg, kernel, args...);  // errors surface at the next synchronising call
     }
 
@@ -870,12 +870,21 @@ struct Launch {
                                   (unsigned)((s.ny + kFlowTY<T> - 1) / kFlowTY<T>) *
                                   (unsigned)((s.nz + chunk - 1) / chunk);
             constexpr int threads = kFlowThreads<T>;
+            // Short CTAs start as those of the kernel before them end; longer ones crowd the
+            // SMs that are done first (us a step of one sweep, early / not: 16^3 16.9 / 18.9,
+            // 40x40x64 26.3 / 27.8, 40x40x192 in chunks of four 39.0 / 38.3, 96x96x512 204.7
+            // / 198.6), and FP64's are long anyway.
+            const bool early = sizeof(T) == 4 && chunk <= 2;
             if (s.units.flow_q == 27) {
-                k_force_march<T, 27><<<grid, threads, 0, st>>>(geo(s), b, F, fc, s.tdev, chunk);
-                k_flow_march<T, 27><<<grid, threads, 0, st>>>(geo(s), dr, u, F, dro, uo, c, s.tdev, chunk);
+                launch_pdl(k_force_march<T, 27>, dim3(grid), dim3(threads), 0, st, early, geo(s), b, F, fc,
+                           (const long long*)s.tdev, chunk, early);
+                launch_pdl(k_flow_march<T, 27>, dim3(grid), dim3(threads), 0, st, early, geo(s), dr, u, (const T*)F, dro,
+                           uo, c, s.tdev, chunk, early);
             } else {
-                k_force_march<T, 19><<<grid, threads, 0, st>>>(geo(s), b, F, fc, s.tdev, chunk);
-                k_flow_march<T, 19><<<grid, threads, 0, st>>>(geo(s), dr, u, F, dro, uo, c, s.tdev, chunk);
+                launch_pdl(k_force_march<T, 19>, dim3(grid), dim3(threads), 0, st, early, geo(s), b, F, fc,
+                           (const long long*)s.tdev, chunk, early);
+                launch_pdl(k_flow_march<T, 19>, dim3(grid), dim3(threads), 0, st, early, geo(s), dr, u, (const T*)F, dro,
+                           uo, c, s.tdev, chunk, early);
             }
         }
         if (s.ib.nm > 0 && s.ib_staged_smem > 0)
