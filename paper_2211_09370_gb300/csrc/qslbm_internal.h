@@ -115,6 +115,7 @@ struct State {
     bool launch_error = false;  // a cudaLaunchKernelEx call failed
     int march_chunk = 16;       // z planes per CTA of the marching sweep (one wave)
     int march_rows = 0;         // rows per thread of the FP32 pair sweep (0: one node per thread)
+    int flow_chunk = 1;         // z planes per CTA of the force and flow kernels
     size_t ib_staged_smem = 0;  // shared memory of k_ib_staged, 0 when it does not fit
     bool ib_early = false;      // k_ib_staged on b may start as the sweep before it ends
     int ib_staged_u = 1;        // its shell nodes per thread per batch of loads (1, 2, 4 or 5)
@@ -184,7 +185,7 @@ struct Ops {
     // s.resident, s.resident_uhalo, s.resident_smem and the kernel's own shape
     // (no allocation)
     cudaError_t (*plan_resident)(State&);
-    cudaError_t (*plan_march)(State&);  // sets s.march_chunk, s.march_rows and s.ib_staged_smem
+    cudaError_t (*plan_march)(State&);  // sets s.march_chunk, s.march_rows, s.flow_chunk and s.ib_staged_smem
     // rows per thread and z planes per CTA of the FP32 pair sweep on a domain that
     // shares the device with share - 1 others
     cudaError_t (*pair_shape)(const State&, int share, int* rows, int* chunk);

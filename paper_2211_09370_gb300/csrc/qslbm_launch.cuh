@@ -93,22 +93,28 @@ struct Launch {
         }
     }
 
-    // Planes per CTA of the marching force and flow kernels: two extra planes are
-    // read per chunk, and a chunk as long as leaves every SM some CTAs hides them.
-    static int flow_chunk(const State& s) {
+    // Planes per CTA of the marching force and flow kernels: two extra planes are read per
+    // chunk, which a chunk as long as fills the device's resident CTAs in few waves hides.
+    static cudaError_t plan_flow(State& s) {
+        if (s.dim != 3) return cudaSuccess;
+        int dev = 0, sms = 0, per_sm = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const void* kern = s.units.flow_q == 27 ? (const void*)k_flow_march<T, 27> : (const void*)k_flow_march<T, 19>;
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFlowThreads<T>, 0);
+        if (e != cudaSuccess) return e;
         const long long tiles = (long long)((s.nx + kFlowTX - 1) / kFlowTX) * ((s.ny + kFlowTY<T> - 1) / kFlowTY<T>);
-        const long long slots = 152LL * 4;
-        int best = 1;
+        const long long slots = (long long)std::max(1, sms) * std::max(1, per_sm);
         long long cost = 1LL << 62;
         for (int chunk = 1; chunk <= 32 && chunk <= s.nz; ++chunk) {
             const long long waves = (tiles * ((s.nz + chunk - 1) / chunk) + slots - 1) / slots;
             const long long c = waves * (chunk + 2);
             if (c < cost) {
                 cost = c;
-                best = chunk;
+                s.flow_chunk = chunk;
             }
         }
-        return best;
+        return cudaSuccess;
     }
 
     static void sweeps(State& s, int nsweeps, cudaStream_t st) {
@@ -650,6 +656,7 @@ struct Launch {
             e = wave_chunk(s, kern, kMarchTX * kMarchTY, kMarchTX, kMarchTY, 4, 1, s.march_chunk);
             s.march_rows = 0;
         }
+        if (e == cudaSuccess) e = plan_flow(s);
         if (e != cudaSuccess) return e;
         // the staged IB corrector, when the plane's shell fits shared memory
         // and the shell nodes' marker lists are padded
@@ -865,7 +872,7 @@ struct Launch {
             k_force_nodes<T, 9><<<blocks, kFlowNodeThreads, 0, st>>>(geo(s), b, F, fc, s.tdev);
             k_flow_nodes<T, 9><<<blocks, kFlowNodeThreads, 0, st>>>(geo(s), dr, u, F, dro, uo, c, s.tdev);
         } else {
-            const int chunk = flow_chunk(s);
+            const int chunk = s.flow_chunk;
             const unsigned grid = (unsigned)((s.nx + kFlowTX - 1) / kFlowTX) *
                                   (unsigned)((s.ny + kFlowTY<T> - 1) / kFlowTY<T>) *
                                   (unsigned)((s.nz + chunk - 1) / chunk);
