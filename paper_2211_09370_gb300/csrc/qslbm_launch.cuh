@@ -150,12 +150,13 @@ struct Launch {
                 T* bout = (T*)s.b[1 - s.bcur];
                 const T* u = (const T*)s.u[s.fcur];
                 if (pair_march(s)) {
-                    const auto kern = pair_kernel(s.bext_xy != nullptr, s.march_rows);
-                    const int ty = 8 * s.march_rows;
-                    const dim3 pgrid((unsigned)((s.nx + 2 * kPairTXP - 1) / (2 * kPairTXP)),
-                                     (unsigned)((s.ny + ty - 1) / ty), (unsigned)((s.nz + chunk - 1) / chunk));
-                    launch_pdl(kern, pgrid, dim3(kPairThreads), 0, st, true, geo(s), (const float*)bin, (float*)bout,
-                               (const float*)u, fcoef(c), chunk);
+                    if constexpr (sizeof(T) == 4) {
+                        const int ty = 8 * s.march_rows;
+                        const dim3 pgrid((unsigned)((s.nx + 2 * kPairTXP - 1) / (2 * kPairTXP)),
+                                         (unsigned)((s.ny + ty - 1) / ty), (unsigned)((s.nz + chunk - 1) / chunk));
+                        launch_pdl(pair_kernel(s.bext_xy != nullptr, s.march_rows), pgrid, dim3(kPairThreads), 0, st,
+                                   true, geo(s), bin, bout, u, c, chunk);
+                    }
                 } else if (s.dim == 3) {
                     if (s.bext_xy)
                         k_sweep_march<T, true><<<mgrid, kMarchTX * kMarchTY, 0, st>>>(geo(s), bin, bout, u, c, chunk);
@@ -595,16 +596,9 @@ struct Launch {
         }
     }
     static auto pair_kernel(bool xy, int rows) {
-        return rows == 1 ? (xy ? k_sweep_march_pair<float, true, 1> : k_sweep_march_pair<float, false, 1>)
-                         : (xy ? k_sweep_march_pair<float, true, 2> : k_sweep_march_pair<float, false, 2>);
+        return rows == 1 ? (xy ? k_sweep_march_pair<T, true, 1> : k_sweep_march_pair<T, false, 1>)
+                         : (xy ? k_sweep_march_pair<T, true, 2> : k_sweep_march_pair<T, false, 2>);
     }
-    static SweepCoef<float> fcoef(const SweepCoef<T>& c) {
-        if constexpr (sizeof(T) == 4)
-            return c;
-        else
-            return SweepCoef<float>{};  // never launched: the pair kernel is FP32 only
-    }
-
     // z planes per CTA such that a grid of tiles of tx x ty columns fills one wave of
     // the kernel's resident CTAs (`share`: of which so many such grids run at a time),
     // at least `least`.
@@ -630,17 +624,20 @@ struct Launch {
     // at least four planes: 7.4, 7.6, 7.7, 7.5).  A grid that would need more than four
     // planes only because of the others keeps four.
     static cudaError_t pair_shape(const State& s, int share, int* rows, int* chunk) {
-        const bool xy = s.bext_xy != nullptr;
-        const void *k1 = (const void*)pair_kernel(xy, 1), *k2 = (const void*)pair_kernel(xy, 2);
-        int c1 = 1, c2 = 1, alone = 1;
-        cudaError_t e = wave_chunk(s, k2, kPairThreads, 2 * kPairTXP, kPairTY<2>, 1, 1, alone);
-        if (e == cudaSuccess) e = wave_chunk(s, k2, kPairThreads, 2 * kPairTXP, kPairTY<2>, 1, share, c2);
-        if (e == cudaSuccess) e = wave_chunk(s, k1, kPairThreads, 2 * kPairTXP, kPairTY<1>, 1, share, c1);
-        c2 = std::min(c2, std::max(alone, 4));
-        // (a grid has at most 65535 tiles of rows)
-        *rows = c2 < 4 && 10 * c1 <= 14 * c2 && s.ny <= 65535LL * kPairTY<1> ? 1 : 2;
-        *chunk = *rows == 1 ? c1 : c2;
-        return e;
+        if constexpr (sizeof(T) == 4) {
+            const bool xy = s.bext_xy != nullptr;
+            const void *k1 = (const void*)pair_kernel(xy, 1), *k2 = (const void*)pair_kernel(xy, 2);
+            int c1 = 1, c2 = 1, alone = 1;
+            cudaError_t e = wave_chunk(s, k2, kPairThreads, 2 * kPairTXP, kPairTY<2>, 1, 1, alone);
+            if (e == cudaSuccess) e = wave_chunk(s, k2, kPairThreads, 2 * kPairTXP, kPairTY<2>, 1, share, c2);
+            if (e == cudaSuccess) e = wave_chunk(s, k1, kPairThreads, 2 * kPairTXP, kPairTY<1>, 1, share, c1);
+            c2 = std::min(c2, std::max(alone, 4));
+            // (a grid has at most 65535 tiles of rows)
+            *rows = c2 < 4 && 10 * c1 <= 14 * c2 && s.ny <= 65535LL * kPairTY<1> ? 1 : 2;
+            *chunk = *rows == 1 ? c1 : c2;
+            return e;
+        }
+        return cudaErrorNotSupported;  // FP64 has no pair sweep
     }
 
     // The marching sweep's planes per CTA and, for pairs, rows per thread.
