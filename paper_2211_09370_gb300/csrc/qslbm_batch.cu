@@ -157,19 +157,6 @@ __global__ void __launch_bounds__(kNodeThreads, (kIbStagedMinBlocks<float, U>))
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kNodeThreads) k_batch_ib(const InstDesc<T>* __restrict__ d,
-                                                           const int* __restrict__ pfirst, int kact, int s) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* sdelta = reinterpret_cast<T*>(smem_raw);
-    const int i = find_inst(pfirst, kact, blockIdx.x);
-    const InstDesc<T>& D = d[i];
-    const int z = blockIdx.x - pfirst[i];
-    T* f = D.b[((D.bpar + s) & 1) ^ 1];
-    const long long n = D.g.n;
-    ib_plane<T>(D.ibm, f, f + n, f + 2 * n, (long long)z * D.g.nx * D.g.ny, D.ibm.zinv ? 0 : z, sdelta);
-}
-
-template <typename T>
 __global__ void __launch_bounds__(kNodeThreads) k_batch_force(const InstDesc<T>* __restrict__ d,
                                                               const int* __restrict__ pfirst, int k) {
     const int i = find_inst(pfirst, k, blockIdx.x);

@@ -59,7 +59,7 @@ struct GroupJob {
     float w0, w1, w1k, sq;
     unsigned base;               // sweeps done before the launch
     int P, GN;                   // nodes of a plane, of the group
-    unsigned mP, mR, mS;         // group_magic of P, R, S
+    unsigned mP, mR, mS;         // magic_of P, R, S
     int abort;
 };
 
@@ -73,13 +73,6 @@ inline long long group_msgs(int P) { return 4LL * P; }
 inline size_t group_smem_bytes(int stride, int R, int S, int E, int G, int P) {
     return 36 * (size_t)stride + 16 * (size_t)(G + 2) + 16 * (size_t)G * R + 8 * ((size_t)9 * R + E + S) +
            4 * ((size_t)R + (P + 31) / 32) + 16;
-}
-
-// t / d for t d < 2^32 as a high multiply, m = group_magic(d) (exact in that
-// range: m d - 2^32 < d).
-__host__ __device__ inline unsigned group_magic(unsigned d) { return d > 1 ? 0xFFFFFFFFu / d + 1u : 0u; }
-__device__ __forceinline__ int group_div(int t, int d, unsigned m) {
-    return d > 1 ? (int)__umulhi((unsigned)t, m) : t;
 }
 
 // XY: some instance has an in-plane applied field (QSLBM_B0_FIELD).
@@ -97,7 +90,7 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
     const int nx = D.g.nx, ny = D.g.ny, nz = D.g.nz;
     const int P = nx * ny, n = (int)D.g.n;
     const int G = gd.G, z0 = gd.z0, GN = G * P;
-    const unsigned mX = group_magic(nx);
+    const unsigned mX = magic_of(nx);
     const bool whole = G == nz;  // the group holds every plane: no exchange
     const int tid = threadIdx.x;
     // the ring and shell of plane 0, which every plane carries (z-invariant tables)
@@ -135,9 +128,9 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
             J.abort = 0;
             J.P = P;
             J.GN = GN;
-            J.mP = group_magic(P);
-            J.mR = group_magic(R);
-            J.mS = group_magic(S);
+            J.mP = magic_of(P);
+            J.mR = magic_of(R);
+            J.mS = magic_of(S);
         }
         for (int t = tid; t < G + 2; t += kGroupThreads) {
             const int zz = t == 0 ? zm : (t == G + 1 ? zp : z0 + t - 1);
@@ -192,7 +185,7 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
             for (int k = 0; k < NPT; ++k) {
                 const int i = tid + k * kGroupThreads;
                 if (i < GN) {
-                    const int g = group_div(i, P, mP);
+                    const int g = magic_div(i, P, mP);
                     const float4 bz = sbz[g + 1];
                     float be[3] = {bz.x, bz.y, bz.z};
                     if constexpr (XY) bext_add_xy(J.bxy, P, i - g * P, be);
@@ -214,7 +207,7 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
             // stay in registers
 #pragma unroll 1
             for (int p = tid; p < P; p += kGroupThreads) {
-                const int y = group_div(p, nx, mX), x = p - y * nx;
+                const int y = magic_div(p, nx, mX), x = p - y * nx;
                 const int dl = x == 0 ? nx - 1 : -1, dr = x == nx - 1 ? 1 - nx : 1;
                 const int du = y == 0 ? P - nx : -nx, dd = y == ny - 1 ? nx - P : nx;
                 const bool now = send && !((shell[p >> 5] >> (p & 31)) & 1u);  // the IB leaves it as it is
@@ -338,7 +331,7 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
             const unsigned seq2 = msg_seq2(J.base + (unsigned)s + 1u);
             uint4* const xo = J.out + (s & 1) * 2 * P;
             for (int t = tid; t < G * R; t += kGroupThreads) {
-                const int g = group_div(t, R, mR), m = t - g * R;
+                const int g = magic_div(t, R, mR), m = t - g * R;
                 const float* f = sn + g * P;
                 float a0 = 0.f, a1 = 0.f, a2 = 0.f;
 #pragma unroll
@@ -356,7 +349,7 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
             __syncthreads();
             // the first and last planes first: their nodes go to the neighbours
             for (int t = tid; t < G * S; t += kGroupThreads) {
-                const int o = group_div(t, S, mS), k = t - o * S;
+                const int o = magic_div(t, S, mS), k = t - o * S;
                 const int g = o == 0 ? 0 : (o == 1 ? G - 1 : o - 1);
                 const int2 node = tsh[k];
                 const float4* dl = sdelta + g * R;

@@ -67,6 +67,13 @@ __device__ __forceinline__ bool wait_counters(const unsigned int* fa, const unsi
     return true;
 }
 
+// t / d for t d < 2^32 as a high multiply, m = magic_of(d) (exact in that range:
+// m d - 2^32 < d).
+__host__ __device__ inline unsigned magic_of(unsigned d) { return d > 1 ? 0xFFFFFFFFu / d + 1u : 0u; }
+__device__ __forceinline__ int magic_div(int t, int d, unsigned m) {
+    return d > 1 ? (int)__umulhi((unsigned)t, m) : t;
+}
+
 // A message: three values and a sequence number in two 64-bit words (a, hi16(b)
 // | seq) and (c, lo16(b) | seq), each of which carries the sequence's low 16
 // bits, so that a reader needs no order between the two words.

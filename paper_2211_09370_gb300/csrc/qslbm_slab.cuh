@@ -126,13 +126,6 @@ struct SlabJob {
     float be[3];
     const float *bext_z, *bext_xy;
 };
-// t / d for t d < 2^32 as a high multiply, m = slab_magic(d) (exact in that
-// range: m d - 2^32 < d).
-__host__ __device__ inline unsigned slab_magic(unsigned d) { return d > 1 ? 0xFFFFFFFFu / d + 1u : 0u; }
-__device__ __forceinline__ int slab_div(int t, int d, unsigned m) {
-    return d > 1 ? (int)__umulhi((unsigned)t, m) : t;
-}
-
 __device__ __forceinline__ float2 slab_mul(float2 a, float2 b) { return mul2(a, b); }
 __device__ __forceinline__ float2 slab_sub(float2 a, float2 b) { return sub2(a, b); }
 __device__ __forceinline__ float2 slab_fma(float2 a, float2 b, float2 c) { return fma2(a, b, c); }
@@ -162,8 +155,8 @@ __device__ __forceinline__ void slab_job_init(SlabJob& J, const SweepCoef<float>
     J.MH = J.MS / 2;
     J.R = ib.ring_off[1] - ib.ring_off[0];
     J.S_ = ib.shell_off[1] - ib.shell_off[0];
-    J.mR = slab_magic((unsigned)J.R);
-    J.mS = slab_magic((unsigned)J.S_);
+    J.mR = magic_of((unsigned)J.R);
+    J.mS = magic_of((unsigned)J.S_);
     J.base = *J.count;
     J.w0 = c.w0;
     J.w1 = c.w1;
@@ -669,7 +662,7 @@ __device__ __forceinline__ void slab_direct(const SlabJob& J, const IBView<float
                 float4* td = t_d();
                 for (int t = tid; t < n3; t += NT) {
                     const int gm = t / 3, a = t - 3 * gm;
-                    const int pg = slab_div(gm, R, mR), m = gm - pg * R;
+                    const int pg = magic_div(gm, R, mR), m = gm - pg * R;
                     const float* f = sb + a * CS + pg * PS;
                     const float2* w = tw + 5 * m;
                     const unsigned* q = tq + 5 * m;
@@ -697,7 +690,7 @@ __device__ __forceinline__ void slab_direct(const SlabJob& J, const IBView<float
                 float *up = J.up, *down = J.down;
                 const float w1 = J.w1;
                 for (int t = tid; t < nS; t += NT) {
-                    const int pg = slab_div(t, S, mS), i = t - pg * S;
+                    const int pg = magic_div(t, S, mS), i = t - pg * S;
                     const float4* dl4 = td + pg * R;
                     const float4 w = tsw[i];
                     const uint4 q = tsm[i];
