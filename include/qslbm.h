@@ -336,8 +336,10 @@ int qslbm_check_bounded_wait(double limit_s, int32_t counter_set, int32_t* gave_
  *    qslbm_batch_handle and the server).  Instances are admitted smallest
  *    first while their groups fit co-resident on the device;
  *  - chains (FP32): every other instance (and any created with sweep_kernel =
- *    QSLBM_SWEEP_SPLIT), when they are at most 24, sweeps in kernels of its
- *    own, several instances at a time on streams of the batch's;
+ *    QSLBM_SWEEP_SPLIT), when they are at most 24 with at most 65536 launches
+ *    a step, sweeps in kernels of its own, several instances at a time on
+ *    streams of the batch's (a server also weighs its chunk of steps against
+ *    capturing their graph anew);
  *  - joint march: otherwise they take one persistent z-marching launch per
  *    sweep over the instances with N_mag > s, then one IB launch; the sweep's
  *    launch mode, tile shape and persistent grid are chosen by timing
@@ -410,7 +412,10 @@ typedef struct qslbm_server qslbm_server;
                                   running requests keep its one launch per step)       */
 
 typedef struct qslbm_server_config {
-    int64_t hbm_budget_bytes; /* device memory the running requests may hold  */
+    int64_t hbm_budget_bytes; /* device memory the running requests' handles may
+                                 hold; the batch's own tables and step graphs
+                                 (1.5 KB a launch, 24 MB at most at N_mag = 270)
+                                 come on top                                   */
     int32_t chunk_steps;      /* flow steps between residual checks            */
     int32_t max_running;      /* 0 = limited by the budget only                */
     int32_t precision;        /* QSLBM_FP32 | QSLBM_FP64 for every request     */

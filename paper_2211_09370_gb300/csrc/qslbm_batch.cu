@@ -461,13 +461,31 @@ void launch_groups(qslbm_batch& B, cudaStream_t st) {
 // 48x48x180 12.7 / 18.3, 9.9, 8.9, 9.1, 9.1; nine 32x32x100 5.0 / 22.7, 13.6, 8.2, 5.5,
 // 3.0 (nine).  One to three members, joint / chains: one 32x32x100 2.12 / 1.46, two 2.28 /
 // 1.91, three 2.88 / 1.85, one 40x40x192 3.02 / 2.34, two 48x48x180 5.23 / 3.32.
+//
+// The graph of a step holds every sweep of every chain, where the joint march has one
+// launch for all: about 1.5 us to capture and instantiate and 1.5 KB of device memory a
+// launch (24 pipes of 40x40x192: 12 963 launches, 543 jointly; at N_mag 1080 51 843, 117 ms
+// more to create and 26 ms of 155 less a step).  Above kChainLaunches a step the batch
+// marches jointly.  A server captures anew whenever its members change, so chains have to
+// earn that back within a chunk of steps (server_chains).
 constexpr int kChains = 24;
+constexpr long long kChainLaunches = 65536;
 constexpr int kChainStreams = 16;
 constexpr long long kChainInFlight = 1200000;
 
 bool chain_member(const State& s) {
     return s.esz == 4 && s.dim == 3 && (s.ib.nm == 0 || s.ib_staged_smem > 0) &&
            s.ny <= 65535LL * qslbm::kPairTY<2>;  // (a grid's tiles of rows; the joint march has one dimension)
+}
+
+// Whether a server's marching members sweep in chains: from five steps a chunk on, or
+// where members of some 0.5 M nodes step long enough.  Ms for requests of 1 to 5 chunks,
+// joint / chains: 20 of 40x40x100 chunk 1 142 / 225, 2 213 / 272, 5 411 / 410, 10 719 /
+// 646; 6 of 48x48x100 chunk 1 59 / 70, 5 190 / 171; 10 of 30x30x60 chunk 2 68 / 99, 5 136 /
+// 129; 2 of 60x60x150 chunk 1 28 / 27; 3 of 80x80x200 chunk 1 85 / 77, 10 429 / 324.
+// work: their nodes times sweeps a step, sweeps: their sweeps a step.
+bool server_chains(int chunk_steps, long long work, long long sweeps) {
+    return chunk_steps >= 5 || (double)chunk_steps * work >= 0.5e6 * sweeps;
 }
 
 void launch_chain(qslbm_batch& B, int k, cudaStream_t st) {
@@ -1015,13 +1033,18 @@ int set_members(qslbm_batch* B, const std::vector<qslbm_handle*>& hs, const std:
     }
     // chains or the joint march, for all marching members alike
     int marching = 0;
+    long long work = 0, sweeps = 0;
     bool chains = B->precision == QSLBM_FP32;
     for (int i = 0; i < count; ++i)
         if (gp[i] == 0) {
+            const State& s = qslbm::handle_state_mut(hs[i]);
             ++marching;
-            chains = chains && chain_member(qslbm::handle_state_mut(hs[i]));
+            sweeps += s.units.n_mag;
+            work += s.n * s.units.n_mag;
+            chains = chains && chain_member(s);
         }
-    chains = chains && marching <= kChains;
+    chains = chains && marching <= kChains && 2 * sweeps <= kChainLaunches;
+    if (!B->owns_members) chains = chains && server_chains(B->chunk_target, work, sweeps);  // (a server's batch)
     std::vector<int> idx(count);
     std::iota(idx.begin(), idx.end(), 0);
     // jointly marching members first, then the chains', then the groups'
