@@ -1261,16 +1261,51 @@ double now_s(const qslbm_server& S) {
     return std::chrono::duration<double>(std::chrono::steady_clock::now() - S.t0).count();
 }
 
-// Groups of the resident group kernel a request would take at the largest
-// group size (-1: the kernel does not hold it: 2-D, no wall, planes above
-// kGroupStrideS nodes).
-int groups_needed(const qslbm_params& p) {
+// Groups of the resident group kernel a request would take at the largest group size
+// for a shared-memory stride (-1: the kernel does not hold it there: 2-D, no wall, planes
+// above the stride).  The large stride leaves little room to the tables, so that their
+// size, from the wall's length, counts there: some 3.5 shell nodes and nine list entries
+// a marker.
+int groups_needed(const qslbm_params& p, int stride, int optin) {
     if (p.dim != 3 || p.geometry == QSLBM_PERIODIC) return -1;
     const long long P = (long long)p.nx * p.ny;
-    if (P > qslbm::kGroupStrideS || p.nz < 1) return -1;
-    const int G = std::max(1, std::min(p.nz, (int)(qslbm::kGroupStrideS / P)));
+    if (P > stride || p.nz < 1) return -1;
+    int G = std::max(1, std::min(p.nz, (int)(stride / P)));
+    if (stride > qslbm::kGroupStrideS) {
+        const double wall = p.geometry == QSLBM_PIPE ? M_PI * p.diameter : 2.0 * p.nx;
+        const int R = (int)std::min(1e6, std::ceil(wall / p.marker_spacing));
+        const int S = (int)std::min<long long>(P, 7LL * R / 2);
+        while (G > 0 && qslbm::group_smem_bytes(stride, R, S, 9 * R, G, (int)P) > (size_t)optin) --G;
+        if (G == 0) return -1;
+    }
     return (p.nz + G - 1) / G;
 }
+
+// The groups that a set of requests takes at either stride, one of which set_members
+// gives them all: the small one counts unless a request is held at the large one only.
+struct GroupsHeld {
+    long long used[2] = {0, 0};
+    bool valid[2] = {true, true};  // every request that either stride holds, this one does
+    void need(const qslbm_params& p, int optin, int n[2]) const {
+        n[0] = groups_needed(p, qslbm::kGroupStrideS, optin);
+        n[1] = groups_needed(p, qslbm::kGroupStrideL, optin);
+    }
+    void add(const qslbm_params& p, int optin) {
+        int n[2];
+        need(p, optin, n);
+        if (n[0] < 0 && n[1] < 0) return;
+        for (int k = 0; k < 2; ++k) {
+            valid[k] = valid[k] && n[k] >= 0;
+            used[k] += std::max(0, n[k]);
+        }
+    }
+    bool fits(const qslbm_params& p, int optin, int cap) const {
+        int n[2];
+        need(p, optin, n);
+        const int k = valid[0] && n[0] >= 0 ? 0 : 1;
+        return valid[k] && n[k] >= 0 && used[k] + n[k] <= cap;
+    }
+};
 
 // Device bytes a request will hold (fields, double buffers, scratch, tables).
 long long estimate_bytes(const qslbm_params& p) {
@@ -1307,10 +1342,11 @@ int server_run(qslbm_server& S, int32_t* n_running, int32_t* n_pending) {
     {
         std::lock_guard<std::mutex> lock(S.mu);
         // smallest first in FP32: keep the running requests within the group
-        // kernel's capacity (a request beyond it would put the whole batch on
-        // the marching route's launches every step)
+        // kernel's capacity (a request beyond it adds two launches a sweep to
+        // every step of the batch)
         const bool hold = S.cfg.admit == QSLBM_ADMIT_SMALLEST && S.cfg.precision == QSLBM_FP32;
-        int used_groups = 0;
+        GroupsHeld held;
+        int optin = 0;
         // a request larger than the whole budget is answered at once
         for (auto it = S.pending.begin(); it != S.pending.end();) {
             if (estimate_bytes(it->p) > S.cfg.hbm_budget_bytes) {
@@ -1332,15 +1368,15 @@ int server_run(qslbm_server& S, int32_t* n_running, int32_t* n_pending) {
             });
             int rc0 = group_capacity(*S.batch);
             if (rc0) return rc0;
-            for (const Running& r : S.running) used_groups += std::max(0, groups_needed(r.r.p));
+            optin = S.batch->goptin;
+            for (const Running& r : S.running) held.add(r.r.p, optin);
         }
         for (auto it = S.pending.begin(); it != S.pending.end();) {
             if (S.cfg.max_running > 0 && (int)S.running.size() >= S.cfg.max_running) break;
             const long long est = estimate_bytes(it->p);
             if (hold) {
-                const int ng = groups_needed(it->p);
-                if (!S.running.empty() && (ng < 0 || used_groups + ng > S.batch->gcap)) break;
-                if (S.used + est <= S.cfg.hbm_budget_bytes) used_groups += std::max(0, ng);
+                if (!S.running.empty() && !held.fits(it->p, optin, S.batch->gcap)) break;
+                if (S.used + est <= S.cfg.hbm_budget_bytes) held.add(it->p, optin);
             }
             if (S.used + est > S.cfg.hbm_budget_bytes) {
                 ++it;
