@@ -77,9 +77,11 @@ extern "C" {
  * same wall ring on every plane; create fails with QSLBM_EINVAL otherwise.
  * AUTO picks RESIDENT when it fits (in FP32 also with several planes per CTA and
  * with an in-plane field, forms that a request for RESIDENT by name does not
- * take); else, when FUSED applies, it times FUSED and SPLIT on the handle's fields at creation (without changing them) and
- * keeps FUSED only when it is at least 2 % faster (the two give bitwise equal
- * results); else SPLIT. */
+ * take, where the domain and the sweeps per step make that the faster route);
+ * else, when FUSED applies, it times FUSED and SPLIT on the handle's fields at
+ * creation (without changing them) and keeps FUSED only when it is at least 2 %
+ * faster (the two give bitwise equal results); else SPLIT.  qslbm_sweep_plan
+ * reports the kernel and its shape. */
 /* Initial velocity: rest (plus the seeded noise), or the Ha = 0 profile
  * U0 (1 - r^2/R^2) along the axis inside the wall (plus the noise). */
 #define QSLBM_INIT_REST 0

@@ -22,7 +22,7 @@
 // EMF form, the staged IB's sums in the same order).
 //
 // What bounds it: the chain of a sweep (e, exchange, walk, markers, shell, with a
-// barrier between each) and shared-memory wavefronts (about 32 a node).  Twelve
+// barrier between each) and shared-memory wavefronts (about 3.3 a node and sweep).  Twelve
 // pipes of 24^2 to 28^2 nodes, 151 groups of up to eight planes: 9.6 us a sweep;
 // with a counter per group (fence, release, acquire, then the halo loads) in place
 // of messages, and u loaded at its use, 10.4 for eleven of them.

@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(kMarchTX* kMarchTY) k_sweep_march(Geo g, const
 // neighbour was a two-way bank conflict).  An even width moves a pair as one
 // 8-byte access; an odd one, whose rows start at odd nodes, as two.  Sweep alone,
 // 96x96x512: 37.2 us against 40.0 with one row per thread and scalar arithmetic
-// (4.6 TB/s of the 36 B a node; 15.8 M warp instructions against 21.4 M), with the
+// (4.6 TB/s of the 36 B a node; 16.5 M warp instructions against 21.4 M), with the
 // IB 49.3 against 51.0; 72x72x384 27.2 against 30.7; 89x89x300 (one scalar node
 // per thread before) 31.7 against 36.5.  (L2 eviction hints on u, b or the new b:
 // 39.8 to 44 us at 96x96x512.)  The joint march of a batch keeps march_tile: small
