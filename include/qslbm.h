@@ -214,7 +214,8 @@ int qslbm_create(const qslbm_params* p, qslbm_handle** out);
 /* Lattice-unit values of the handle.  Errors: QSLBM_EINVAL (NULL argument). */
 int qslbm_get_units(const qslbm_handle* h, qslbm_units* out);
 
-/* The kernel that runs a handle's magnetic sweeps, and its shape.
+/* The kernel that runs a handle's magnetic sweeps, and its shape (of a batch
+ * member's handle: what it would run by itself).
  *   kernel   QSLBM_KERNEL_*
  *   ctas     CTAs of a launch
  *   threads  threads per CTA
